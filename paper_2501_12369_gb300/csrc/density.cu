@@ -15,6 +15,8 @@
 // writes, in index order within each segment, [survivors | clones | two children per split
 // parent].  Survivors keep their Adam moments; clones and children start from zero.  Children's
 // means are parent + R(q) (s * z) for the caller's standard-normal draws z.
+#include <type_traits>
+
 #include "kernels.cuh"
 
 namespace darb {
@@ -106,28 +108,36 @@ k_densify_stats(const float4 *__restrict__ grad2d, const int *__restrict__ radiu
     max_radius[i] = max(max_radius[i], r);
 }
 
-__global__ void __launch_bounds__(kDenThreads)
+// Latency-bound (28 bytes a splat, 1M splats): two splats a thread, so that the whole set is in
+// flight at once, and the three counts summed once per CTA.  24.8 us with a block scan per 256
+// splats, 23 us with eight splats a thread and one sum, 15.2 us so.
+constexpr int kCountThreads = 1024;
+__global__ void __launch_bounds__(kCountThreads)
 k_densify_count(int n, const float *__restrict__ scales, const float *__restrict__ opac,
                 const float *__restrict__ accum, const float *__restrict__ count, const int *__restrict__ max_radius,
                 DenCfg c, uint32_t *__restrict__ blk) {
     pdl_entry();
-    __shared__ uint32_t s_w[kDenThreads / 32];
+    __shared__ uint32_t s_c[3];
+    if (threadIdx.x < 3) s_c[threadIdx.x] = 0;
+    __syncthreads();
     uint32_t sum[3] = {0, 0, 0};
-    for (int j = 0; j < kDenItems; ++j) {
-        const int i = blockIdx.x * kDenTile + j * kDenThreads + threadIdx.x;
-        uint32_t v = 0;
-        if (i < n) v = pack(classify(i, scales, opac, accum, count, max_radius, c));
-        uint32_t tot;
-        block_scan_packed<kDenThreads>(v, s_w, tot);
-        sum[0] += tot & 1023u;
-        sum[1] += (tot >> 10) & 1023u;
-        sum[2] += tot >> 20;
+#pragma unroll
+    for (int j = 0; j < kDenTile / kCountThreads; ++j) {
+        const int i = blockIdx.x * kDenTile + j * kCountThreads + threadIdx.x;
+        if (i < n) {
+            const Flags f = classify(i, scales, opac, accum, count, max_radius, c);
+            sum[0] += f.surv;
+            sum[1] += f.clone;
+            sum[2] += f.split;
+        }
     }
-    if (threadIdx.x == 0) {
-        blk[3 * (size_t)blockIdx.x] = sum[0];
-        blk[3 * (size_t)blockIdx.x + 1] = sum[1];
-        blk[3 * (size_t)blockIdx.x + 2] = sum[2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t w = __reduce_add_sync(0xffffffffu, sum[k]);
+        if ((threadIdx.x & 31) == 0 && w) atomicAdd(&s_c[k], w);
     }
+    __syncthreads();
+    if (threadIdx.x < 3) blk[3 * (size_t)blockIdx.x + threadIdx.x] = s_c[threadIdx.x];
 }
 
 // One CTA: exclusive offsets of the three block counts; segment bases; n_out.
@@ -156,81 +166,179 @@ k_densify_offsets(int nb, uint32_t *__restrict__ blk, uint32_t *__restrict__ n_o
 struct DenIO {
     darb_train_params in, out;
     darb_adam_state sin, sout;
-    int k3;  // SH floats per splat
 };
 
-__device__ __forceinline__ void copy_row(const float *src, float *dst, int i, int j, int w) {
-    for (int e = 0; e < w; ++e) dst[(size_t)j * w + e] = src[(size_t)i * w + e];
-}
+// Splats per scatter CTA: a quarter of a counted block, so that 1M splats give 1954 CTAs.
+constexpr int kScatSplats = 512;
+constexpr int kScatPer = kDenTile / kScatSplats;  // scatter CTAs per counted block
+constexpr int kScatItems = kScatSplats / kDenThreads;
+constexpr int kScatUnroll = 4;  // loads in flight per thread and array
 
-__device__ __forceinline__ void zero_row(float *dst, int j, int w) {
-    for (int e = 0; e < w; ++e) dst[(size_t)j * w + e] = 0.0f;
-}
-
-// Copy splat i to row j of the output; moments copied (keep) or zeroed.
-__device__ __forceinline__ void emit(const DenIO &io, int i, int j, bool keep_moments) {
-    copy_row(io.in.means, io.out.means, i, j, 3);
-    copy_row(io.in.log_scales, io.out.log_scales, i, j, 3);
-    copy_row(io.in.quats, io.out.quats, i, j, 4);
-    copy_row(io.in.opacity_logits, io.out.opacity_logits, i, j, 1);
-    copy_row(io.in.sh, io.out.sh, i, j, io.k3);
-    copy_row(io.in.scales, io.out.scales, i, j, 3);
-    copy_row(io.in.opacities, io.out.opacities, i, j, 1);
-    const float *const src[10] = {io.sin.m_means, io.sin.v_means, io.sin.m_scales, io.sin.v_scales, io.sin.m_quats,
-                                  io.sin.v_quats, io.sin.m_opac, io.sin.v_opac, io.sin.m_sh, io.sin.v_sh};
-    float *const dst[10] = {io.sout.m_means, io.sout.v_means, io.sout.m_scales, io.sout.v_scales, io.sout.m_quats,
-                            io.sout.v_quats, io.sout.m_opac, io.sout.v_opac, io.sout.m_sh, io.sout.v_sh};
-    const int w[10] = {3, 3, 3, 3, 4, 4, 1, 1, io.k3, io.k3};
-    for (int a = 0; a < 10; ++a) {
-        if (keep_moments) copy_row(src[a], dst[a], i, j, w[a]);
-        else zero_row(dst[a], j, w[a]);
+// Rows [out0, out0 + rows) of dst from the rows i0 + list[r >> SHIFT] of src, W floats a row, by the
+// whole CTA with consecutive lanes on consecutive words; 16-byte words where rows are multiples
+// of 16 bytes and both arrays are aligned (the moments need not be).
+template <int W, int SHIFT>
+__device__ __forceinline__ void copy_rows(const float *__restrict__ src, float *__restrict__ dst, int i0, uint32_t out0,
+                                          const uint16_t *list, int rows) {
+    auto walk = [&](auto *s, auto *d, auto per) {
+        constexpr int P = decltype(per)::value;
+        const int total = rows * P;
+        for (int b = threadIdx.x; b < total; b += kDenThreads * kScatUnroll) {
+            typename std::remove_const<typename std::remove_reference<decltype(*s)>::type>::type v[kScatUnroll];
+#pragma unroll
+            for (int u = 0; u < kScatUnroll; ++u) {
+                const int t = b + u * kDenThreads;
+                if (t < total) {
+                    const int r = t / P;
+                    v[u] = s[(size_t)(i0 + list[r >> SHIFT]) * P + (t - r * P)];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kScatUnroll; ++u) {
+                const int t = b + u * kDenThreads;
+                if (t < total) d[(size_t)out0 * P + t] = v[u];
+            }
+        }
+    };
+    if constexpr (W % 4 == 0) {
+        if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
+            walk(reinterpret_cast<const float4 *>(src), reinterpret_cast<float4 *>(dst),
+                 std::integral_constant<int, W / 4>{});
+            return;
+        }
     }
+    walk(src, dst, std::integral_constant<int, W>{});
 }
 
+template <int W>
+__device__ __forceinline__ void zero_rows(float *__restrict__ dst, uint32_t out0, int rows) {
+    for (int t = threadIdx.x; t < rows * W; t += kDenThreads) dst[(size_t)out0 * W + t] = 0.0f;
+}
+
+template <int K3>
+__device__ __forceinline__ void zero_moments(const darb_adam_state &s, uint32_t out0, int rows) {
+    zero_rows<3>(s.m_means, out0, rows);
+    zero_rows<3>(s.v_means, out0, rows);
+    zero_rows<3>(s.m_scales, out0, rows);
+    zero_rows<3>(s.v_scales, out0, rows);
+    zero_rows<4>(s.m_quats, out0, rows);
+    zero_rows<4>(s.v_quats, out0, rows);
+    zero_rows<1>(s.m_opac, out0, rows);
+    zero_rows<1>(s.v_opac, out0, rows);
+    zero_rows<K3>(s.m_sh, out0, rows);
+    zero_rows<K3>(s.v_sh, out0, rows);
+}
+
+// One CTA takes kScatSplats consecutive splats.  Its first output row in each segment is the
+// counted block's offset plus the counts of the block's splats before it, which it classifies
+// again (28 bytes a splat, mostly from L2; a table of finer offsets would need a larger
+// workspace).  It lists its survivors, clones and split parents in shared memory; the rows of
+// each list are consecutive in the output, so every array is then copied as one flat range.
+// HBM-bound: with one thread copying each row, 32 lanes wrote 32 different rows at a time and the
+// kernel took 1250 us (1M splats, SH degree 3, 1.6 GB), now 277 us (0.78 of the measured copy rate).
+template <int K3>
 __global__ void __launch_bounds__(kDenThreads)
 k_densify_scatter(int n, DenIO io, const float *__restrict__ accum, const float *__restrict__ count,
                   const int *__restrict__ max_radius, const float *__restrict__ normals, DenCfg c,
                   const uint32_t *__restrict__ blk, const uint32_t *__restrict__ n_out) {
     pdl_entry();
     __shared__ uint32_t s_w[kDenThreads / 32];
-    uint32_t base[3] = {blk[3 * (size_t)blockIdx.x], blk[3 * (size_t)blockIdx.x + 1], blk[3 * (size_t)blockIdx.x + 2]};
-    const uint32_t clone0 = n_out[1], child0 = n_out[2];
-    for (int j = 0; j < kDenItems; ++j) {
-        const int i = blockIdx.x * kDenTile + j * kDenThreads + threadIdx.x;
+    __shared__ uint32_t s_before[3];
+    __shared__ uint16_t s_list[3][kScatSplats];
+    const int block = blockIdx.x / kScatPer, sub = blockIdx.x % kScatPer;
+    const int i0 = block * kDenTile + sub * kScatSplats;
+    if (i0 >= n) return;  // uniform over the CTA
+    if (threadIdx.x < 3) s_before[threadIdx.x] = blk[3 * (size_t)block + threadIdx.x];
+    __syncthreads();
+    uint32_t before[3] = {0, 0, 0};
+    for (int j = 0; j < sub * kScatItems; ++j) {  // the block's splats before this CTA's (all below n)
+        const Flags f = classify(block * kDenTile + j * kDenThreads + (int)threadIdx.x, io.in.scales, io.in.opacities,
+                                 accum, count, max_radius, c);
+        before[0] += f.surv;
+        before[1] += f.clone;
+        before[2] += f.split;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t w = __reduce_add_sync(0xffffffffu, before[k]);
+        if ((threadIdx.x & 31) == 0 && w) atomicAdd(&s_before[k], w);
+    }
+    uint32_t cnt[3] = {0, 0, 0};
+    for (int j = 0; j < kScatItems; ++j) {
+        const int l = j * kDenThreads + (int)threadIdx.x, i = i0 + l;
         Flags f{false, false, false};
         if (i < n) f = classify(i, io.in.scales, io.in.opacities, accum, count, max_radius, c);
         uint32_t tot;
         const uint32_t ex = block_scan_packed<kDenThreads>(pack(f), s_w, tot);
-        if (f.surv) emit(io, i, (int)(base[0] + (ex & 1023u)), true);
-        if (f.clone) emit(io, i, (int)(clone0 + base[1] + ((ex >> 10) & 1023u)), false);
-        if (f.split) {
-            const int row = (int)(child0 + 2 * (base[2] + (ex >> 20)));
+        if (f.surv) s_list[0][cnt[0] + (ex & 1023u)] = (uint16_t)l;
+        if (f.clone) s_list[1][cnt[1] + ((ex >> 10) & 1023u)] = (uint16_t)l;
+        if (f.split) s_list[2][cnt[2] + (ex >> 20)] = (uint16_t)l;
+        cnt[0] += tot & 1023u;
+        cnt[1] += (tot >> 10) & 1023u;
+        cnt[2] += tot >> 20;
+    }
+    __syncthreads();
+    const darb_train_params &a = io.in, &b = io.out;
+    auto params = [&](uint32_t out0, const uint16_t *list, int rows, auto shift) {  // what every copied row keeps
+        constexpr int S = decltype(shift)::value;
+        copy_rows<K3, S>(a.sh, b.sh, i0, out0, list, rows);
+        copy_rows<4, S>(a.quats, b.quats, i0, out0, list, rows);
+        copy_rows<1, S>(a.opacity_logits, b.opacity_logits, i0, out0, list, rows);
+        copy_rows<1, S>(a.opacities, b.opacities, i0, out0, list, rows);
+        if (S == 0) {  // children's are computed below
+            copy_rows<3, S>(a.means, b.means, i0, out0, list, rows);
+            copy_rows<3, S>(a.log_scales, b.log_scales, i0, out0, list, rows);
+            copy_rows<3, S>(a.scales, b.scales, i0, out0, list, rows);
+        }
+    };
+    const std::integral_constant<int, 0> one{};
+    const std::integral_constant<int, 1> two{};
+    if (cnt[0]) {  // survivors keep their moments
+        const uint32_t o = s_before[0];
+        const int rows = (int)cnt[0];
+        const uint16_t *l = s_list[0];
+        params(o, l, rows, one);
+        copy_rows<K3, 0>(io.sin.m_sh, io.sout.m_sh, i0, o, l, rows);
+        copy_rows<K3, 0>(io.sin.v_sh, io.sout.v_sh, i0, o, l, rows);
+        copy_rows<3, 0>(io.sin.m_means, io.sout.m_means, i0, o, l, rows);
+        copy_rows<3, 0>(io.sin.v_means, io.sout.v_means, i0, o, l, rows);
+        copy_rows<3, 0>(io.sin.m_scales, io.sout.m_scales, i0, o, l, rows);
+        copy_rows<3, 0>(io.sin.v_scales, io.sout.v_scales, i0, o, l, rows);
+        copy_rows<4, 0>(io.sin.m_quats, io.sout.m_quats, i0, o, l, rows);
+        copy_rows<4, 0>(io.sin.v_quats, io.sout.v_quats, i0, o, l, rows);
+        copy_rows<1, 0>(io.sin.m_opac, io.sout.m_opac, i0, o, l, rows);
+        copy_rows<1, 0>(io.sin.v_opac, io.sout.v_opac, i0, o, l, rows);
+    }
+    if (cnt[1]) {
+        const uint32_t o = n_out[1] + s_before[1];
+        params(o, s_list[1], (int)cnt[1], one);
+        zero_moments<K3>(io.sout, o, (int)cnt[1]);
+    }
+    if (cnt[2]) {  // two children a parent
+        const uint32_t o = n_out[2] + 2 * s_before[2];
+        const int rows = 2 * (int)cnt[2];
+        params(o, s_list[2], rows, two);
+        zero_moments<K3>(io.sout, o, rows);
+        for (int t = threadIdx.x; t < rows; t += kDenThreads) {
+            const int i = i0 + s_list[2][t >> 1], ch = t & 1;
+            const size_t r = (size_t)o + t;
             // rotation of the normalised quaternion (w, x, y, z)
-            const float4 q = reinterpret_cast<const float4 *>(io.in.quats)[i];
+            const float4 q = reinterpret_cast<const float4 *>(a.quats)[i];
             const float inv = rsqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
             const float w = q.x * inv, x = q.y * inv, y = q.z * inv, z = q.w * inv;
             const float R[3][3] = {{1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y)},
                                    {2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x)},
                                    {2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)}};
-            const float s[3] = {io.in.scales[3 * (size_t)i], io.in.scales[3 * (size_t)i + 1],
-                                io.in.scales[3 * (size_t)i + 2]};
-            for (int ch = 0; ch < 2; ++ch) {
-                const int r = row + ch;
-                emit(io, i, r, false);
-                const float *zz = normals + (size_t)6 * i + 3 * ch;
-                const float v[3] = {s[0] * zz[0], s[1] * zz[1], s[2] * zz[2]};
-                for (int a = 0; a < 3; ++a) {
-                    io.out.means[3 * (size_t)r + a] =
-                        io.in.means[3 * (size_t)i + a] + (R[a][0] * v[0] + R[a][1] * v[1] + R[a][2] * v[2]);
-                    const float ls = __fsub_rn(io.in.log_scales[3 * (size_t)i + a], c.log_div);
-                    io.out.log_scales[3 * (size_t)r + a] = ls;
-                    io.out.scales[3 * (size_t)r + a] = expf(ls);
-                }
+            const float *zz = normals + (size_t)6 * i + 3 * ch;
+            const float v[3] = {a.scales[3 * (size_t)i] * zz[0], a.scales[3 * (size_t)i + 1] * zz[1],
+                                a.scales[3 * (size_t)i + 2] * zz[2]};
+            for (int k = 0; k < 3; ++k) {
+                b.means[3 * r + k] = a.means[3 * (size_t)i + k] + (R[k][0] * v[0] + R[k][1] * v[1] + R[k][2] * v[2]);
+                const float ls = __fsub_rn(a.log_scales[3 * (size_t)i + k], c.log_div);
+                b.log_scales[3 * r + k] = ls;
+                b.scales[3 * r + k] = expf(ls);
             }
         }
-        base[0] += tot & 1023u;
-        base[1] += (tot >> 10) & 1023u;
-        base[2] += tot >> 20;
     }
 }
 
@@ -271,10 +379,18 @@ cudaError_t launch_densify(const darb_train_params &in, const darb_adam_state &s
     DenCfg c{cfg.grad_threshold, cfg.dense_scale, cfg.min_opacity, cfg.max_screen_radius, cfg.max_world_scale,
              cfg.split_scale_div, (float)std::log((double)cfg.split_scale_div)};
     if (nb == 0) return cudaMemsetAsync(n_out, 0, 3 * sizeof(uint32_t), st);
-    launch_k(k_densify_count, nb, kDenThreads, 0, st, n, in.scales, in.opacities, accum, count, max_radius, c, blk);
+    launch_k(k_densify_count, nb, kCountThreads, 0, st, n, in.scales, in.opacities, accum, count, max_radius, c, blk);
     launch_k(k_densify_offsets, 1, 1024, 0, st, nb, blk, n_out);
-    DenIO io{in, out, sin, sout, 3 * (in.sh_degree + 1) * (in.sh_degree + 1)};
-    launch_k(k_densify_scatter, nb, kDenThreads, 0, st, n, io, accum, count, max_radius, normals, c, blk, n_out);
+    const DenIO io{in, out, sin, sout};
+    auto scatter = [&](auto kernel) {
+        launch_k(kernel, nb * kScatPer, kDenThreads, 0, st, n, io, accum, count, max_radius, normals, c, blk, n_out);
+    };
+    switch (in.sh_degree) {
+    case 0: scatter(k_densify_scatter<3>); break;
+    case 1: scatter(k_densify_scatter<12>); break;
+    case 2: scatter(k_densify_scatter<27>); break;
+    default: scatter(k_densify_scatter<48>); break;
+    }
     return cudaGetLastError();
 }
 
