@@ -183,7 +183,9 @@ darb_status darb_render_batch(const darb_splats *splats, const darb_camera *cams
     // host-side descriptors, then their upload through kernel parameters
     std::vector<BatchView> hv(V);
     int total_tiles = 0;
+    bool aux = false;
     for (int v = 0; v < V; ++v) {
+        aux |= outs[v].last || outs[v].n_contrib;
         unsigned char *vb = w + L.views + L.per_view * (size_t)v;
         const ProjectedOut po = view_projected(vb, n);
         const int tx = tile_count(cams[v].width, tile), ty = tile_count(cams[v].height, tile);
@@ -253,7 +255,7 @@ darb_status darb_render_batch(const darb_splats *splats, const darb_camera *cams
         if (cudaEventRecord(P.join[s], P.side[s]) != cudaSuccess) return DARB_ERR_CUDA;
         if (cudaStreamWaitEvent(st, P.join[s], 0) != cudaSuccess) return DARB_ERR_CUDA;
     }
-    if (launch_render_fwd_batch(kparams->kind, tile, desc, V, total_tiles, queue, kparams->q_max,
+    if (launch_render_fwd_batch(kparams->kind, tile, desc, V, total_tiles, aux, queue, kparams->q_max,
                                 kparams->q_max_strict ? 1 : 0, make_spec(*kparams), bp->max_ctas, st) != cudaSuccess)
         return DARB_ERR_CUDA;
     return DARB_OK;

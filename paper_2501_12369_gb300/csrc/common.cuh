@@ -123,8 +123,39 @@ __device__ __forceinline__ float sinc_series(float u) {
     return __fmaf_rn(r, -u, 1.0f);
 }
 
+// The approximate instructions with subnormals flushed (.ftz): without the flag each carries three
+// more instructions that rescale a subnormal operand or result, and no argument here is one.
+// Checked against __expf, __cosf, __fdividef and rsqrtf for every float q in [0, 9]: the same bits.
+__device__ __forceinline__ float ex2_ftz(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// sqrt(q) by one Newton step in the residual form s + (q - s^2) / (2 sqrt(q)) with a fused
+// residual (Markstein, IBM J. Res. Dev. 34, 1990) from the approximate root; checked against
+// __fsqrt_rn for every float in (1e-30, 9]: the same bits, at a third of the instructions.
+// Smaller q give 1e-15, whose profile is the profile at 0.
+__device__ __forceinline__ float sqrt_newton(float q) {
+    const float c = fmaxf(q, 1e-30f), r = rsqrt_ftz(c);
+    float s;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(c));
+    return __fmaf_rn(__fmaf_rn(-s, s, c), __fmul_rn(0.5f, r), s);
+}
+
+// exp(-q / 2) = 2^(-q / (2 ln 2))
+constexpr float kHalfLog2e = 0.72134752044448170368f;
 template <> __device__ __forceinline__ float kernel_F<DARB_GAUSSIAN>(float q, const KernelSpec &) {
-    return __expf(__fmul_rn(-0.5f, q));
+    return ex2_ftz(__fmul_rn(q, -kHalfLog2e));
 }
 template <> __device__ __forceinline__ float kernel_dF<DARB_GAUSSIAN>(float q, const KernelSpec &) { return -0.5f * __expf(-0.5f * q); }
 
@@ -136,7 +167,7 @@ template <> __device__ __forceinline__ float kernel_dF<DARB_HALF_COSINE>(float q
 }
 
 template <> __device__ __forceinline__ float kernel_F<DARB_RAISED_COSINE>(float q, const KernelSpec &) {
-    return __fmaf_rn(0.5f, __cosf(__fmul_rn(__fsqrt_rn(q), kPi / 2.5f)), 0.5f);
+    return __fmaf_rn(0.5f, __cosf(__fmul_rn(sqrt_newton(q), kPi / 2.5f)), 0.5f);
 }
 template <> __device__ __forceinline__ float kernel_dF<DARB_RAISED_COSINE>(float q, const KernelSpec &) {
     // -(k/4) sin(k sqrt q) / sqrt q, k = pi/2.5; limit -k^2/4 at q = 0.
@@ -164,7 +195,7 @@ template <> __device__ __forceinline__ float kernel_dF<DARB_MOD_SINC>(float q, c
 }
 
 template <> __device__ __forceinline__ float kernel_F<DARB_INV_QUADRIC>(float q, const KernelSpec &) {
-    return __fdividef(1.0f, __fadd_rn(1.0f, q));
+    return rcp_ftz(__fadd_rn(1.0f, q));
 }
 template <> __device__ __forceinline__ float kernel_dF<DARB_INV_QUADRIC>(float q, const KernelSpec &) {
     const float r = __fdividef(1.0f, 1.0f + q);
@@ -172,7 +203,7 @@ template <> __device__ __forceinline__ float kernel_dF<DARB_INV_QUADRIC>(float q
 }
 
 template <> __device__ __forceinline__ float kernel_F<DARB_INV_MULTIQUADRIC>(float q, const KernelSpec &) {
-    return rsqrtf(__fadd_rn(1.0f, q));
+    return rsqrt_ftz(__fadd_rn(1.0f, q));
 }
 template <> __device__ __forceinline__ float kernel_dF<DARB_INV_MULTIQUADRIC>(float q, const KernelSpec &) {
     const float r = rsqrtf(1.0f + q);

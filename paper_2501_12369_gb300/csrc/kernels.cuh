@@ -50,8 +50,8 @@ struct BatchView {
 };
 
 // render.cu: persistent launch over all views' tiles; queue is a device counter (reset here).
-// max_ctas > 0 caps the grid (else SMs x resident CTAs).
-cudaError_t launch_render_fwd_batch(int kind, int tile, const BatchView *views, int n_views, int total_tiles,
+// max_ctas > 0 caps the grid (else SMs x resident CTAs).  aux: some view has a last or n_contrib buffer.
+cudaError_t launch_render_fwd_batch(int kind, int tile, const BatchView *views, int n_views, int total_tiles, bool aux,
                                     uint32_t *queue, float qmax, int strict, const KernelSpec &ks, int max_ctas,
                                     cudaStream_t st);
 

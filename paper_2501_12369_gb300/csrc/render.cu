@@ -2,11 +2,11 @@
 // splat run (paper Sec. 4.1 "alpha blending ... similar to 3DGS", Eq. HalfCosine and
 // Eq. 2DSplattedFunction; forward and backward listings of Sec. B).
 //
-// One CTA per tile.  Each thread owns PIX pixels of one column of the tile (rows r, r + TILE/PIX,
-// ...), so every splat record loaded from shared memory serves PIX pixels and dx is shared.  The
+// A CTA takes a tile (backward) or a square of one (forward).  Each thread owns PIX pixels of one
+// column, so every splat record loaded from shared memory serves PIX pixels and dx is shared.  The
 // tile's run is consumed in batches of NT records (NT = threads): each thread gathers one splat's
 // record (mean, conic, opacity, colour) into shared memory, then every thread walks the batch.  A
-// CTA-wide vote ends the loop once every pixel of the tile has stopped (T < 1e-4) -- the early
+// CTA-wide vote ends the loop once every pixel of the CTA has stopped (T < 1e-4) -- the early
 // termination of 3DGS.
 //
 // The support test uses the fixed FP32 sequence conic_q(), and alpha / the kernel value are
@@ -24,15 +24,32 @@ struct Bg {
 
 constexpr int kMaxDevicesRender = 64;
 
-#ifndef DARB_FWD_PIX32
-#define DARB_FWD_PIX32 4
-#endif
-template <int TILE>
-struct RenderShape {
-    static constexpr int PIX = TILE == 32 ? DARB_FWD_PIX32 : (TILE >= 16 ? 2 : 1);  // pixels per thread
-    static constexpr int NT = TILE * TILE / PIX;      // threads per CTA = records per batch
-    static constexpr int ROWS = TILE / PIX;           // row stride between a thread's pixels
+// The forward's CTA composites a SUB x SUB square of a tile (the squares of a tile walk the same
+// list), PIX pixels a thread.  A warp covers a compact block (LX columns, LY * PIX rows), because it
+// walks until its last pixel has stopped and neighbouring pixels stop at about the same record; a
+// thread's pixels share their column, so that dx is shared.
+template <int TILE_, int SUB_, int PIX_>
+struct FwdShape {
+    static constexpr int TILE = TILE_, SUB = SUB_, PIX = PIX_;
+    static constexpr int NT = SUB * SUB / PIX;  // threads per CTA = records per batch
+    static constexpr int PARTS = (TILE / SUB) * (TILE / SUB);
+    static constexpr int LX = SUB == 32 || (SUB == 16 && PIX == 4) ? 16 : 8, LY = 32 / LX;
+    static constexpr int BH = LY * PIX, BX = SUB / LX;  // rows of a warp's block, blocks side by side
+    static_assert(BH <= SUB && SUB % BH == 0, "blocks tile the square");
+    __device__ static int column() { return (int)((threadIdx.x >> 5) % BX) * LX + (int)(threadIdx.x & 31) % LX; }
+    __device__ static int row(int k) {
+        return (int)((threadIdx.x >> 5) / BX) * BH + (int)(threadIdx.x & 31) / LX + k * LY;
+    }
 };
+// 16 x 16 squares (8 x 8 in 8-pixel tiles, one warp) of two pixels a thread.  A CTA holds its place
+// until its slowest warp has stopped, so small squares cost less although each gathers its records
+// again: Gaussian, 1M splats, 1080p, 32-pixel tiles: 169 us with the whole tile as one CTA of four
+// pixels a thread, 152 with squares of 16 and four pixels, 148 with two, 162 with squares of 8;
+// 8-pixel tiles 155 us with one pixel a thread, 118 with two.
+template <int TILE> struct FwdOf { using S = FwdShape<TILE, TILE == 8 ? 8 : 16, 2>; };
+// The batched launch takes four pixels a thread (2026 us against 2096 for 16 views of 1M splats:
+// its views' lists are short and half the warps then fetch items and records).
+template <int TILE> struct BatchOf { using S = FwdShape<TILE, TILE == 8 ? 8 : 16, TILE == 8 ? 2 : 4>; };
 
 // Resident CTAs per SM the compositing kernels may be compiled for (a register budget);
 // unset, the compiler chooses.  The backward compiles to 64 registers under a budget of 3 or
@@ -40,11 +57,6 @@ struct RenderShape {
 // 0.186 ms against 0.190 for the half-cosine at 3M / 1080p (Gaussian 0.604 against 0.612).
 #ifndef DARB_BWD_MIN_CTAS
 #define DARB_BWD_MIN_CTAS 3
-#endif
-#ifdef DARB_FWD_MIN_CTAS
-#define DARB_FWD_BOUNDS(nt) __launch_bounds__(nt, DARB_FWD_MIN_CTAS)
-#else
-#define DARB_FWD_BOUNDS(nt) __launch_bounds__(nt)
 #endif
 #ifdef DARB_BWD_MIN_CTAS
 #define DARB_BWD_BOUNDS(nt) __launch_bounds__(nt, DARB_BWD_MIN_CTAS)
@@ -59,54 +71,78 @@ struct RenderShape {
 #endif
 template <int TILE>
 struct BwdShape {
-    static constexpr int PIX = TILE == 32 ? DARB_BWD_PIX32 : RenderShape<TILE>::PIX;
+    static constexpr int PIX = TILE == 32 ? DARB_BWD_PIX32 : (TILE == 16 ? 2 : 1);
     static constexpr int NT = TILE * TILE / PIX;
     static constexpr int ROWS = TILE / PIX;
 };
 
-// The forward's per-pair body: branch-free, a pair that does not blend taking weight 0 (1), or
-// one branch per failed test (0).  Both give the same bits: C + rgb * 0 = C and T is kept.
-// Branch-free measured 0.108 -> 0.103 ms (half-cosine) at 3M splats / 1080p.  The backward
-// keeps its branches: there a pair that does not contribute would still pay for F', the
-// reciprocal and the nine products (0.204 -> 0.212 ms half-cosine, 0.669 -> 0.736 Gaussian).
-// Both passes test the support against support_limit(q_max, strict), taken once per thread:
-// with the strictness a kernel argument tested per pair, the forward took 0.103 ms and the
-// backward 0.204 ms (half-cosine), against 0.089 and 0.190 ms.
-#ifndef DARB_FWD_SELECT
-#define DARB_FWD_SELECT 1
-#endif
+// Lane arithmetic on one value or on a pair (the packed two-lane FP32 instructions of sm_100+, which
+// round each lane as the scalar form does).
+template <int L> struct Lanes;
+template <> struct Lanes<1> {
+    using T = float;
+    static __device__ __forceinline__ T dup(float a) { return a; }
+    static __device__ __forceinline__ T mul(T a, T b) { return __fmul_rn(a, b); }
+    static __device__ __forceinline__ T add(T a, T b) { return __fadd_rn(a, b); }
+    static __device__ __forceinline__ T fma(T a, T b, T c) { return __fmaf_rn(a, b, c); }
+    static __device__ __forceinline__ float &at(T &v, int) { return v; }
+};
+template <> struct Lanes<2> {
+    using T = float2;
+    static __device__ __forceinline__ T dup(float a) { return make_float2(a, a); }
+    static __device__ __forceinline__ T mul(T a, T b) { return __fmul2_rn(a, b); }
+    static __device__ __forceinline__ T add(T a, T b) { return __fadd2_rn(a, b); }
+    static __device__ __forceinline__ T fma(T a, T b, T c) { return __ffma2_rn(a, b, c); }
+    static __device__ __forceinline__ float &at(T &v, int l) { return l ? v.y : v.x; }
+};
 
-// A batch of staged records: the 9 floats of a splat in two float4s and a float (1), so that a
-// thread reads a record in 3 shared-memory loads, or as mean, conic + opacity and colour (0).
-// Packed measured 0.0886 -> 0.0846 ms (half-cosine) and 0.306 -> 0.293 ms (Gaussian) at 3M
-// splats / 1080p.  Folding a pixel's saturation into the branch-free predicate instead of
-// skipping it by a branch was mixed (+2% half-cosine, -2% Gaussian) and is not done.  The
-// backward keeps its three arrays: packed, its red and green stay live across the pixel loop
-// (65-71 registers, 3 CTAs per SM), 0.187 -> 0.193 ms (half-cosine), 0.603 -> 0.621 (Gaussian).
-#ifndef DARB_FWD_PACK
-#define DARB_FWD_PACK 1
-#endif
+// kernel_F on every lane: the multiplications in front of the special functions, and the whole sinc
+// series, on pairs.  The same operations as kernel_F, so the same bits.
+template <int KIND, int L>
+__device__ __forceinline__ typename Lanes<L>::T kernel_F_lanes(typename Lanes<L>::T q, const KernelSpec &ks) {
+    using V = Lanes<L>;
+    typename V::T r = q;
+    if constexpr (KIND == DARB_GAUSSIAN || KIND == DARB_HALF_COSINE) {
+        r = V::mul(q, V::dup(KIND == DARB_GAUSSIAN ? -kHalfLog2e : kPi / 18.0f));
+#pragma unroll
+        for (int l = 0; l < L; ++l) V::at(r, l) = KIND == DARB_GAUSSIAN ? ex2_ftz(V::at(r, l)) : __cosf(V::at(r, l));
+    } else if constexpr (KIND == DARB_PARABOLA) {
+        r = V::fma(q, V::dup(-1.0f / 9.0f), V::dup(1.0f));
+    } else if constexpr (KIND == DARB_MOD_SINC) {
+        const typename V::T u = V::mul(q, V::dup(kPi * kPi / 9.0f));
+        r = V::fma(u, V::dup(1.0f / 1307674368000.0f), V::dup(-1.0f / 6227020800.0f));
+        r = V::fma(r, u, V::dup(1.0f / 39916800.0f));
+        r = V::fma(r, u, V::dup(-1.0f / 362880.0f));
+        r = V::fma(r, u, V::dup(1.0f / 5040.0f));
+        r = V::fma(r, u, V::dup(-1.0f / 120.0f));
+        r = V::fma(r, u, V::dup(1.0f / 6.0f));
+        r = V::fma(r, V::mul(u, V::dup(-1.0f)), V::dup(1.0f));
+#pragma unroll
+        for (int l = 0; l < L; ++l) V::at(r, l) = fmaxf(V::at(r, l), 0.0f);
+    } else {
+#pragma unroll
+        for (int l = 0; l < L; ++l) V::at(r, l) = kernel_F<KIND>(V::at(q, l), ks);
+    }
+    return r;
+}
 
-// The forward's branch-free body on pairs of a thread's pixels with the packed two-lane FP32
-// instructions of sm_100+ (1), or one pixel at a time (0).  The backward keeps one pixel at a
-// time: paired (a pair with one contributing lane costing what one pixel does), it needed 80
-// registers and 3 CTAs per SM and measured 0.195 against 0.186 ms (half-cosine), also with
-// each warp's pixels in 4 consecutive rows so that more pairs have both lanes contributing.
-#ifndef DARB_FWD_PAIR
-#define DARB_FWD_PAIR 1
-#endif
+// Records walked per step of the forward: their alphas do not depend on the transmittance, so a
+// step's alphas overlap; a batch is padded with records of opacity 0 to whole steps.
+// Steps of 4 records and few resident threads (512 an SM, up to 128 registers) for the plain forward:
+// overlap within a warp pays more than more warps (157 us against 169 at steps of 2 and 768
+// threads, 188 at steps of 1 and 1024, Gaussian).  The L1 forward is a training step's, whose
+// dense scenes stop after some 20 records: steps of 2 and 1024 threads, as its CTAs mostly wait on
+// their gathers.  The batched launch: 2 and 768.
+constexpr int kStepPlain = 4, kStepL1 = 2, kStepBatch = 2;
+constexpr int kThreadsPlain = 512, kThreadsL1 = 1024, kThreadsBatch = 768;  // resident per SM at least
 
-template <int TILE>
+// A batch of staged records: the 9 floats of a splat in two float4s and a float, so that a thread
+// reads a record in 3 shared-memory loads.
+template <int NT>
 struct FwdSmem {
-#if DARB_FWD_PACK
-    float4 a[RenderShape<TILE>::NT];  // x, y, A, 2B
-    float4 b[RenderShape<TILE>::NT];  // C, opacity, red, green
-    float c[RenderShape<TILE>::NT];   // blue
-#else
-    float2 xy[RenderShape<TILE>::NT];
-    float4 co[RenderShape<TILE>::NT];  // A, 2B, C, opacity
-    float rgb[RenderShape<TILE>::NT][3];
-#endif
+    float4 a[NT];  // x, y, A, 2B
+    float4 b[NT];  // C, opacity, red, green
+    float c[NT];   // blue
 };
 
 // Where a tile's results go; t_final, last and n_contrib may be null (not written).
@@ -130,187 +166,119 @@ struct L1Out {
 
 // One tile of one view, by the whole CTA.  sink() is called once, after the compositing loop,
 // so the output pointers need not stay live in registers across it.  With L1 the epilogue also
-// takes the L1 loss of the tile's pixels (every thread of the CTA reaches it).
-template <int KIND, int TILE, bool L1 = false, class SinkFn>
-__device__ __forceinline__ void render_tile_fwd(int tile, FwdSmem<TILE> &sm, const uint2 *__restrict__ ranges,
+// takes the L1 loss of the tile's pixels (every thread of the CTA reaches it).  AUX: the outputs
+// beside the image and T that the caller may ask for (0: none, 1: last, 2: last and n_contrib).
+//
+// The body is branch-free and keeps few instructions on the ALU pipe (compares, selects, minimum),
+// which runs at half the rate of the FP32 pipe and bound it before.  For every (pixel, record),
+// with the support and alpha tests in `use`:
+//   a = use ? alpha : 0;  t' = t (1 - a);  blend = use and t' >= 1e-4
+//   w = blend ? a t : 0;  T = blend ? t' : T;  t = t'
+// t runs on past the stop, where it stays below 1e-4 as every factor is at most 1, so a stopped
+// pixel needs no flag of its own, and the chain from record to record is one multiplication.  A
+// record that does not blend leaves t, T and the colours exactly as they are.  q >= 0 and
+// q <= q_lim are one unsigned comparison (q is never -0: it ends in an addition to +0 or more).
+// Pairs of records instead of pairs of pixels as the packed lanes (no value then needs duplicating)
+// took as many instructions and more registers (189 us against 175 at the time).
+template <int KIND, class S, int AUX, int STEP, bool L1 = false, class SinkFn>
+__device__ __forceinline__ void render_tile_fwd(int item, FwdSmem<S::NT> &sm,
+                                                const uint2 *__restrict__ ranges,
                                                 const uint32_t *__restrict__ values,
                                                 const float2 *__restrict__ mean2d,
                                                 const float4 *__restrict__ conic_o, const float *__restrict__ rgb,
                                                 int W, int H, int tiles_x, float qmax, int strict,
                                                 const KernelSpec &ks, SinkFn sink, const L1Out &l1 = L1Out{},
                                                 float *s_l1 = nullptr) {
-    using S = RenderShape<TILE>;
-    constexpr int NT = S::NT, PIX = S::PIX;
-    const int tx = tile % tiles_x, ty = tile / tiles_x;
-    const int px = tx * TILE + (threadIdx.x % TILE);
-    const int py0 = ty * TILE + (threadIdx.x / TILE);
+    constexpr int TILE = S::TILE, NT = S::NT, PIX = S::PIX, L = PIX % 2 == 0 ? 2 : 1, NV = PIX / L;  // NV groups of L lanes
+    using V = Lanes<L>;
+    using VT = typename V::T;
+    static_assert(NT % STEP == 0, "a full batch is whole steps");
+    const int tile = item / S::PARTS, part = item % S::PARTS;
+    const int px = (tile % tiles_x) * TILE + part % (TILE / S::SUB) * S::SUB + S::column();
+    const int y0 = (tile / tiles_x) * TILE + part / (TILE / S::SUB) * S::SUB;
     const float fpx = (float)px + 0.5f;
     const uint2 r = ranges[tile];
     const int start = (int)r.x, end = (int)r.y;
-    const float qlim = support_limit(qmax, strict);
+    const uint32_t qlim = __float_as_uint(support_limit(qmax, strict));
 
-    float fpy[PIX], T[PIX], C0[PIX], C1[PIX], C2[PIX];
+    VT t[NV], Tf[NV], C0[NV], C1[NV], C2[NV], nfpy[NV];
     uint32_t count[PIX], lastp[PIX];
-    bool done[PIX];
 #pragma unroll
-    for (int k = 0; k < PIX; ++k) {
-        const int py = py0 + k * S::ROWS;
-        fpy[k] = (float)py + 0.5f;
-        T[k] = 1.0f;
-        C0[k] = C1[k] = C2[k] = 0.0f;
-        count[k] = lastp[k] = 0;
-        done[k] = !(px < W && py < H);
-    }
-    // pixels 2p and 2p + 1 as the lanes of one pair (the packed FP32 instructions)
-    constexpr bool kPair = DARB_FWD_PAIR && DARB_FWD_SELECT && PIX % 2 == 0;
-    constexpr int NPP = PIX / 2 > 0 ? PIX / 2 : 1;
-    float2 T2[NPP], C0p[NPP], C1p[NPP], C2p[NPP], nfpy[NPP];
+    for (int v = 0; v < NV; ++v) {
+        Tf[v] = V::dup(1.0f);
+        C0[v] = C1[v] = C2[v] = V::dup(0.0f);
 #pragma unroll
-    for (int pp = 0; pp < NPP; ++pp) {
-        T2[pp] = make_float2(1.0f, 1.0f);
-        C0p[pp] = C1p[pp] = C2p[pp] = make_float2(0.0f, 0.0f);
-        nfpy[pp] = make_float2(-fpy[(2 * pp) % PIX], -fpy[(2 * pp + 1) % PIX]);
+        for (int l = 0; l < L; ++l) {
+            const int py = y0 + S::row(v * L + l);
+            V::at(nfpy[v], l) = -((float)py + 0.5f);
+            V::at(t[v], l) = px < W && py < H ? 1.0f : 0.0f;  // pixels outside the image have stopped
+            count[v * L + l] = lastp[v * L + l] = 0;
+        }
     }
+    auto all_stopped = [&] {
+        float m = 0.0f;
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+            for (int l = 0; l < L; ++l) m = fmaxf(m, V::at(t[v], l));
+        return m < kTMin;
+    };
     for (int b0 = start; b0 < end; b0 += NT) {
-        bool all_done = true;
-#pragma unroll
-        for (int k = 0; k < PIX; ++k) all_done &= done[k];
-        if (__syncthreads_count(all_done) == NT) break;
-        const int idx = b0 + (int)threadIdx.x;
-        if (idx < end) {
-            const uint32_t id = values[idx];
+        const bool stopped = all_stopped();
+        if (__syncthreads_count(stopped) == NT) break;
+        const int nb = min(NT, end - b0), i = threadIdx.x;
+        if (i < nb) {
+            const uint32_t id = values[b0 + i];
             const float2 xy = mean2d[id];
-            float4 co = conic_o[id];
-            co.y = 2.0f * co.y;
+            const float4 co = conic_o[id];
             const float c0 = rgb[3 * (size_t)id], c1 = rgb[3 * (size_t)id + 1], c2 = rgb[3 * (size_t)id + 2];
-#if DARB_FWD_PACK
-            sm.a[threadIdx.x] = make_float4(xy.x, xy.y, co.x, co.y);
-            sm.b[threadIdx.x] = make_float4(co.z, co.w, c0, c1);
-            sm.c[threadIdx.x] = c2;
-#else
-            sm.xy[threadIdx.x] = xy;
-            sm.co[threadIdx.x] = co;
-            sm.rgb[threadIdx.x][0] = c0;
-            sm.rgb[threadIdx.x][1] = c1;
-            sm.rgb[threadIdx.x][2] = c2;
-#endif
+            sm.a[i] = make_float4(xy.x, xy.y, co.x, 2.0f * co.y);
+            sm.b[i] = make_float4(co.z, co.w, c0, c1);
+            sm.c[i] = c2;
+        } else if (i < nb + STEP) {  // the last step's padding
+            sm.a[i] = sm.b[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            sm.c[i] = 0.0f;
         }
         __syncthreads();
-        if (all_done) continue;
-        const int nb = min(NT, end - b0);
-        for (int j = 0; j < nb; ++j) {
-#if DARB_FWD_PACK
-            const float4 pa = sm.a[j], pb = sm.b[j];
-            const float2 xy = make_float2(pa.x, pa.y);
-            const float4 co = make_float4(pa.z, pa.w, pb.x, pb.y);
-            const float r0 = pb.z, r1 = pb.w, r2 = sm.c[j];
-#else
-            const float2 xy = sm.xy[j];
-            const float4 co = sm.co[j];
-            const float r0 = sm.rgb[j][0], r1 = sm.rgb[j][1], r2 = sm.rgb[j][2];
-#endif
-            const float dx = __fsub_rn(xy.x, fpx);
-            bool any_live = false;
-            if constexpr (kPair) {
-                // the scalar branch-free body below on pairs of pixels: every paired operation
-                // rounds per lane as its scalar form (__fmul_rn, __fmaf_rn, 1 - alpha), so the
-                // support decisions and the sums are the same bits
-                const uint32_t pos = (uint32_t)(b0 - start + j + 1);
-                const float2 dx2 = make_float2(dx, dx), y2 = make_float2(xy.y, xy.y);
-                const float2 A2 = make_float2(co.x, co.x), B2 = make_float2(co.y, co.y);
-                const float2 Cc2 = make_float2(co.z, co.z), o2 = make_float2(co.w, co.w);
-                const float2 one2 = make_float2(1.0f, 1.0f);
+        if (stopped) continue;
+        const uint32_t pos0 = (uint32_t)(b0 - start + 1);
+        for (int j0 = 0; j0 < nb; j0 += STEP) {
 #pragma unroll
-                for (int pp = 0; pp < NPP; ++pp) {
-                    const int k0 = 2 * pp, k1 = 2 * pp + 1;
-                    if (done[k0] && done[k1]) continue;
-                    any_live = true;
-                    const float2 dy = __fadd2_rn(y2, nfpy[pp]);
-                    const float2 g = __ffma2_rn(A2, dx2, __fmul2_rn(B2, dy));
-                    const float2 q = __ffma2_rn(dx2, g, __fmul2_rn(__fmul2_rn(Cc2, dy), dy));
-                    const float2 of = __fmul2_rn(o2, make_float2(kernel_F<KIND>(q.x, ks), kernel_F<KIND>(q.y, ks)));
-                    const float2 alpha = make_float2(fminf(kAlphaMax, of.x), fminf(kAlphaMax, of.y));
-                    const float2 Tn = __fmul2_rn(T2[pp], __fadd2_rn(one2, make_float2(-alpha.x, -alpha.y)));
-                    const bool use0 = !done[k0] && in_support_lim(q.x, qlim) && alpha.x >= kAlphaMin;
-                    const bool use1 = !done[k1] && in_support_lim(q.y, qlim) && alpha.y >= kAlphaMin;
-                    const bool stop0 = Tn.x < kTMin, stop1 = Tn.y < kTMin;
-                    if (use0 && stop0) done[k0] = true;
-                    if (use1 && stop1) done[k1] = true;
-                    const bool blend0 = use0 && !stop0, blend1 = use1 && !stop1;
-                    const float2 wp = __fmul2_rn(alpha, T2[pp]);
-                    const float2 w = make_float2(blend0 ? wp.x : 0.0f, blend1 ? wp.y : 0.0f);
-                    C0p[pp] = __ffma2_rn(make_float2(r0, r0), w, C0p[pp]);
-                    C1p[pp] = __ffma2_rn(make_float2(r1, r1), w, C1p[pp]);
-                    C2p[pp] = __ffma2_rn(make_float2(r2, r2), w, C2p[pp]);
-                    T2[pp] = make_float2(blend0 ? Tn.x : T2[pp].x, blend1 ? Tn.y : T2[pp].y);
-                    count[k0] += blend0 ? 1u : 0u;
-                    count[k1] += blend1 ? 1u : 0u;
-                    lastp[k0] = blend0 ? pos : lastp[k0];
-                    lastp[k1] = blend1 ? pos : lastp[k1];
+            for (int u = 0; u < STEP; ++u) {
+                const float4 pa = sm.a[j0 + u], pb = sm.b[j0 + u];
+                const float pc = sm.c[j0 + u];
+                const VT dx = V::dup(__fsub_rn(pa.x, fpx)), y = V::dup(pa.y), A = V::dup(pa.z), B2 = V::dup(pa.w);
+                const VT Cc = V::dup(pb.x), o = V::dup(pb.y), r0 = V::dup(pb.z), r1 = V::dup(pb.w), r2 = V::dup(pc);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    const VT dy = V::add(y, nfpy[v]);
+                    const VT g = V::fma(A, dx, V::mul(B2, dy));  // conic_q
+                    VT q = V::fma(dx, g, V::mul(V::mul(Cc, dy), dy));
+                    VT a = V::mul(o, kernel_F_lanes<KIND, L>(q, ks));
+                    bool use[L];
+#pragma unroll
+                    for (int l = 0; l < L; ++l) {
+                        const float alpha = fminf(kAlphaMax, V::at(a, l));
+                        use[l] = __float_as_uint(V::at(q, l)) <= qlim && alpha >= kAlphaMin;
+                        V::at(a, l) = use[l] ? alpha : 0.0f;
+                    }
+                    VT w = V::mul(a, t[v]);
+                    t[v] = V::mul(t[v], V::fma(a, V::dup(-1.0f), V::dup(1.0f)));
+#pragma unroll
+                    for (int l = 0; l < L; ++l) {
+                        const float tn = V::at(t[v], l);
+                        const bool blend = use[l] && tn >= kTMin;
+                        V::at(w, l) = blend ? V::at(w, l) : 0.0f;
+                        V::at(Tf[v], l) = blend ? tn : V::at(Tf[v], l);
+                        if (AUX >= 2) count[v * L + l] += blend ? 1u : 0u;
+                        if (AUX >= 1) lastp[v * L + l] = blend ? pos0 + (uint32_t)(j0 + u) : lastp[v * L + l];
+                    }
+                    C0[v] = V::fma(r0, w, C0[v]);
+                    C1[v] = V::fma(r1, w, C1[v]);
+                    C2[v] = V::fma(r2, w, C2[v]);
                 }
-                if (!any_live) break;
-                continue;
             }
-#if DARB_FWD_SELECT
-            const uint32_t pos = (uint32_t)(b0 - start + j + 1);
-#pragma unroll
-            for (int k = 0; k < PIX; ++k) {
-                if (done[k]) continue;
-                any_live = true;
-                const float dy = __fsub_rn(xy.y, fpy[k]);
-                const float q = conic_q(dx, dy, co.x, co.y, co.z);
-                const float alpha = fminf(kAlphaMax, __fmul_rn(co.w, kernel_F<KIND>(q, ks)));
-                const float Tn = T[k] * (1.0f - alpha);
-                const bool use = in_support_lim(q, qlim) && alpha >= kAlphaMin;
-                const bool stop = Tn < kTMin;
-                if (use && stop) done[k] = true;
-                const bool blend = use && !stop;
-                const float w = blend ? alpha * T[k] : 0.0f;  // weight 0 leaves C and T exactly as they are
-                C0[k] = fmaf(r0, w, C0[k]);
-                C1[k] = fmaf(r1, w, C1[k]);
-                C2[k] = fmaf(r2, w, C2[k]);
-                T[k] = blend ? Tn : T[k];
-                count[k] += blend ? 1u : 0u;
-                lastp[k] = blend ? pos : lastp[k];
-            }
-#else
-#pragma unroll
-            for (int k = 0; k < PIX; ++k) {
-                if (done[k]) continue;
-                any_live = true;
-                const float dy = __fsub_rn(xy.y, fpy[k]);
-                const float q = conic_q(dx, dy, co.x, co.y, co.z);
-                if (!in_support_lim(q, qlim)) continue;
-                const float alpha = fminf(kAlphaMax, __fmul_rn(co.w, kernel_F<KIND>(q, ks)));
-                if (alpha < kAlphaMin) continue;
-                const float Tn = T[k] * (1.0f - alpha);
-                if (Tn < kTMin) {
-                    done[k] = true;
-                    continue;
-                }
-                const float w = alpha * T[k];
-                C0[k] = fmaf(r0, w, C0[k]);
-                C1[k] = fmaf(r1, w, C1[k]);
-                C2[k] = fmaf(r2, w, C2[k]);
-                T[k] = Tn;
-                ++count[k];
-                lastp[k] = (uint32_t)(b0 - start + j + 1);
-            }
-#endif
-            if (!any_live) break;
-        }
-    }
-    if constexpr (kPair) {
-#pragma unroll
-        for (int pp = 0; pp < NPP; ++pp) {
-            T[2 * pp] = T2[pp].x;
-            T[2 * pp + 1] = T2[pp].y;
-            C0[2 * pp] = C0p[pp].x;
-            C0[2 * pp + 1] = C0p[pp].y;
-            C1[2 * pp] = C1p[pp].x;
-            C1[2 * pp + 1] = C1p[pp].y;
-            C2[2 * pp] = C2p[pp].x;
-            C2[2 * pp + 1] = C2p[pp].y;
+            if (all_stopped()) break;
         }
     }
     const size_t plane = (size_t)W * H;
@@ -318,10 +286,12 @@ __device__ __forceinline__ void render_tile_fwd(int tile, FwdSmem<TILE> &sm, con
     float acc = 0.0f;  // the pixels' |C - target| (with L1)
 #pragma unroll
     for (int k = 0; k < PIX; ++k) {
-        const int py = py0 + k * S::ROWS;
+        const int py = y0 + S::row(k);
         if (!(px < W && py < H)) continue;
         const size_t pix = (size_t)py * W + px;
-        const float c[3] = {fmaf(T[k], o.bg.r, C0[k]), fmaf(T[k], o.bg.g, C1[k]), fmaf(T[k], o.bg.b, C2[k])};
+        const float T = V::at(Tf[k / L], k % L);
+        const float c[3] = {fmaf(T, o.bg.r, V::at(C0[k / L], k % L)), fmaf(T, o.bg.g, V::at(C1[k / L], k % L)),
+                            fmaf(T, o.bg.b, V::at(C2[k / L], k % L))};
 #pragma unroll
         for (int ch = 0; ch < 3; ++ch) {
             if (o.image) o.image[ch * plane + pix] = c[ch];
@@ -331,9 +301,9 @@ __device__ __forceinline__ void render_tile_fwd(int tile, FwdSmem<TILE> &sm, con
                 acc += fabsf(d);
             }
         }
-        if (o.t_final) o.t_final[pix] = T[k];
-        if (o.last) o.last[pix] = lastp[k];
-        if (o.n_contrib) o.n_contrib[pix] = count[k];
+        if (o.t_final) o.t_final[pix] = T;
+        if (AUX >= 1 && o.last) o.last[pix] = lastp[k];
+        if (AUX >= 2 && o.n_contrib) o.n_contrib[pix] = count[k];
     }
     if constexpr (L1) {
 #pragma unroll
@@ -348,40 +318,42 @@ __device__ __forceinline__ void render_tile_fwd(int tile, FwdSmem<TILE> &sm, con
     }
 }
 
-template <int KIND, int TILE, bool L1>
-__global__ void DARB_FWD_BOUNDS(RenderShape<TILE>::NT)
+template <int KIND, int TILE, int AUX, bool L1>
+__global__ void __launch_bounds__(FwdOf<TILE>::S::NT, (L1 ? kThreadsL1 : kThreadsPlain) / FwdOf<TILE>::S::NT)
 k_render_fwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ values,
              const float2 *__restrict__ mean2d, const float4 *__restrict__ conic_o,
              const float *__restrict__ rgb, int W, int H, int tiles_x, float qmax, int strict, KernelSpec ks, Bg bg,
              float *__restrict__ image, float *__restrict__ t_final, uint32_t *__restrict__ last,
              uint32_t *__restrict__ n_contrib, L1Out l1) {
     pdl_entry();
-    __shared__ FwdSmem<TILE> sm;
-    __shared__ float s_l1[L1 ? RenderShape<TILE>::NT / 32 : 1];
-    render_tile_fwd<KIND, TILE, L1>(blockIdx.x, sm, ranges, values, mean2d, conic_o, rgb, W, H, tiles_x, qmax, strict,
-                                    ks, [&] { return FwdSink{image, t_final, last, n_contrib, bg}; }, l1, s_l1);
+    using S = typename FwdOf<TILE>::S;
+    __shared__ FwdSmem<S::NT> sm;
+    __shared__ float s_l1[L1 ? (S::NT + 31) / 32 : 1];
+    render_tile_fwd<KIND, S, AUX, L1 ? kStepL1 : kStepPlain, L1>(
+        blockIdx.x, sm, ranges, values, mean2d, conic_o, rgb, W, H, tiles_x, qmax, strict, ks,
+        [&] { return FwdSink{image, t_final, last, n_contrib, bg}; }, l1, s_l1);
 }
 
-// Several views in one persistent launch: CTAs take (view, tile) items from a device counter
-// (items numbered view-major; views[v].tile_begin is the first item of view v) until all are
-// done, so small and large views share the GPU without per-view launches or tails.
-template <int KIND, int TILE>
-__global__ void __launch_bounds__(RenderShape<TILE>::NT,
-                                  (RenderShape<TILE>::PIX >= 4 ? 1024 : 1536) / RenderShape<TILE>::NT)
+// Several views in one persistent launch: CTAs take items (a square of a tile of a view) from a
+// device counter (numbered view-major; views[v].tile_begin is the first tile of view v) until all
+// are done, so small and large views share the GPU without per-view launches or tails.
+template <int KIND, int TILE, int AUX>
+__global__ void __launch_bounds__(BatchOf<TILE>::S::NT, kThreadsBatch / BatchOf<TILE>::S::NT)
 k_render_fwd_batch(const BatchView *__restrict__ views, int n_views, int total_tiles, uint32_t *__restrict__ queue,
                    float qmax, int strict, KernelSpec ks) {
     pdl_entry();
-    __shared__ FwdSmem<TILE> sm;
+    using S = typename BatchOf<TILE>::S;
+    __shared__ FwdSmem<S::NT> sm;
     __shared__ int s_item, s_view;
     for (;;) {
         if (threadIdx.x == 0) {
-            const int item = (int)atomicAdd(queue, 1u);
+            const int item = (int)atomicAdd(queue, 1u), t = item / S::PARTS;
             int v = 0;
-            if (item < total_tiles) {  // last view whose first item is <= item
+            if (t < total_tiles) {  // last view whose first tile is <= t
                 int lo = 0, hi = n_views - 1;
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
-                    if (views[mid].tile_begin <= item) lo = mid; else hi = mid - 1;
+                    if (views[mid].tile_begin <= t) lo = mid; else hi = mid - 1;
                 }
                 v = lo;
             }
@@ -390,14 +362,14 @@ k_render_fwd_batch(const BatchView *__restrict__ views, int n_views, int total_t
         }
         __syncthreads();
         const int item = s_item, v = s_view;
-        if (item >= total_tiles) break;
+        if (item / S::PARTS >= total_tiles) break;
         const BatchView &bv = views[v];
-        render_tile_fwd<KIND, TILE>(item - bv.tile_begin, sm, bv.ranges, bv.values, bv.mean2d, bv.conic_o, bv.rgb,
-                                    bv.W, bv.H, bv.tiles_x, qmax, strict, ks, [&] {
-                                        const BatchView &b = views[v];
-                                        return FwdSink{b.image, b.t_final, b.last, b.n_contrib,
-                                                       Bg{b.bg[0], b.bg[1], b.bg[2]}};
-                                    });
+        render_tile_fwd<KIND, S, AUX, kStepBatch>(
+            item - bv.tile_begin * S::PARTS, sm, bv.ranges, bv.values, bv.mean2d, bv.conic_o, bv.rgb, bv.W, bv.H,
+            bv.tiles_x, qmax, strict, ks, [&] {
+                const BatchView &b = views[v];
+                return FwdSink{b.image, b.t_final, b.last, b.n_contrib, Bg{b.bg[0], b.bg[1], b.bg[2]}};
+            });
         __syncthreads();  // the CTA is done with s_item and the staging arrays
     }
 }
@@ -599,14 +571,14 @@ cudaError_t fwd_t(int n_tiles, const uint2 *ranges, const uint32_t *values, cons
                   const float4 *conic_o, const float *rgb, const Cam &cam, int tiles_x, float qmax, int strict,
                   const KernelSpec &ks, float *image, float *t_final, uint32_t *last, uint32_t *n_contrib,
                   const L1Out &l1, cudaStream_t st) {
-    if (l1.target)
-        launch_k(k_render_fwd<KIND, TILE, true>, n_tiles, RenderShape<TILE>::NT, 0, st,
-                 ranges, values, mean2d, conic_o, rgb, cam.W, cam.H, tiles_x, qmax, strict, ks,
-                 Bg{cam.bg[0], cam.bg[1], cam.bg[2]}, image, t_final, last, n_contrib, l1);
-    else
-        launch_k(k_render_fwd<KIND, TILE, false>, n_tiles, RenderShape<TILE>::NT, 0, st,
-                 ranges, values, mean2d, conic_o, rgb, cam.W, cam.H, tiles_x, qmax, strict, ks,
-                 Bg{cam.bg[0], cam.bg[1], cam.bg[2]}, image, t_final, last, n_contrib, l1);
+    using S = typename FwdOf<TILE>::S;
+    auto go = [&](auto kernel) {
+        launch_k(kernel, n_tiles * S::PARTS, S::NT, 0, st, ranges, values, mean2d, conic_o, rgb, cam.W, cam.H,
+                 tiles_x, qmax, strict, ks, Bg{cam.bg[0], cam.bg[1], cam.bg[2]}, image, t_final, last, n_contrib, l1);
+    };
+    if (!l1.target) go(k_render_fwd<KIND, TILE, 2, false>);
+    else if (n_contrib) go(k_render_fwd<KIND, TILE, 2, true>);
+    else go(k_render_fwd<KIND, TILE, 1, true>);
     return cudaGetLastError();
 }
 
@@ -659,17 +631,17 @@ cudaError_t launch_render_fwd(int kind, int tile, int tiles_x, int tiles_y, cons
 
 namespace {
 
-template <int KIND, int TILE>
-cudaError_t fwd_batch_t(const BatchView *views, int n_views, int total_tiles, uint32_t *queue, float qmax, int strict,
-                        const KernelSpec &ks, int max_ctas, cudaStream_t st) {
+template <int KIND, int TILE, int AUX>
+cudaError_t fwd_batch_aux(const BatchView *views, int n_views, int total_tiles, uint32_t *queue, float qmax, int strict,
+                          const KernelSpec &ks, int max_ctas, cudaStream_t st) {
+    constexpr int NT = BatchOf<TILE>::S::NT;
     static int per_sm[kMaxDevicesRender] = {};  // resident CTAs per SM, once per device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     int occ = (dev >= 0 && dev < kMaxDevicesRender) ? per_sm[dev] : 0;
     if (occ == 0) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_render_fwd_batch<KIND, TILE>,
-                                                          RenderShape<TILE>::NT, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_render_fwd_batch<KIND, TILE, AUX>, NT, 0);
         if (e != cudaSuccess) return e;
         occ = occ > 0 ? occ : 1;
         if (dev >= 0 && dev < kMaxDevicesRender) per_sm[dev] = occ;
@@ -679,21 +651,29 @@ cudaError_t fwd_batch_t(const BatchView *views, int n_views, int total_tiles, ui
     if (e != cudaSuccess) return e;
     long long grid = (long long)sms * occ;
     if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
-    if (grid > total_tiles) grid = total_tiles;
+    const long long items = (long long)total_tiles * BatchOf<TILE>::S::PARTS;
+    if (grid > items) grid = items;
     e = launch_zero(st, queue, sizeof(uint32_t));
     if (e != cudaSuccess) return e;
-    launch_k(k_render_fwd_batch<KIND, TILE>, (int)grid, RenderShape<TILE>::NT, 0, st, views, n_views, total_tiles, queue,
-             qmax, strict, ks);
+    launch_k(k_render_fwd_batch<KIND, TILE, AUX>, (int)grid, NT, 0, st, views, n_views, total_tiles, queue, qmax, strict,
+             ks);
     return cudaGetLastError();
+}
+
+template <int KIND, int TILE>
+cudaError_t fwd_batch_t(const BatchView *views, int n_views, int total_tiles, bool aux, uint32_t *queue, float qmax,
+                        int strict, const KernelSpec &ks, int max_ctas, cudaStream_t st) {
+    return aux ? fwd_batch_aux<KIND, TILE, 2>(views, n_views, total_tiles, queue, qmax, strict, ks, max_ctas, st)
+               : fwd_batch_aux<KIND, TILE, 0>(views, n_views, total_tiles, queue, qmax, strict, ks, max_ctas, st);
 }
 
 }  // namespace
 
-cudaError_t launch_render_fwd_batch(int kind, int tile, const BatchView *views, int n_views, int total_tiles,
+cudaError_t launch_render_fwd_batch(int kind, int tile, const BatchView *views, int n_views, int total_tiles, bool aux,
                                     uint32_t *queue, float qmax, int strict, const KernelSpec &ks, int max_ctas,
                                     cudaStream_t st) {
     if (total_tiles == 0 || n_views == 0) return cudaSuccess;
-#define FB_CALL(K, T) fwd_batch_t<K, T>(views, n_views, total_tiles, queue, qmax, strict, ks, max_ctas, st)
+#define FB_CALL(K, T) fwd_batch_t<K, T>(views, n_views, total_tiles, aux, queue, qmax, strict, ks, max_ctas, st)
     if (tile == 8) {
         switch (kind) {
         case 0: return FB_CALL(0, 8); case 1: return FB_CALL(1, 8); case 2: return FB_CALL(2, 8);
