@@ -109,7 +109,6 @@ inline KernelSpec make_spec(const darb_kernel_params &k) {
 }
 
 template <int K> __device__ __forceinline__ float kernel_F(float q, const KernelSpec &ks);
-template <int K> __device__ __forceinline__ float kernel_dF(float q, const KernelSpec &ks);
 
 // sin(x)/x = 1 - u/3! + u^2/5! - ... - u^7/15! with u = x^2, evaluated by Horner as
 // 1 - u (1/3! - u (1/5! - u (1/7! - u (1/9! - u (1/11! - u (1/13! - u/15!)))))).
@@ -157,63 +156,37 @@ constexpr float kHalfLog2e = 0.72134752044448170368f;
 template <> __device__ __forceinline__ float kernel_F<DARB_GAUSSIAN>(float q, const KernelSpec &) {
     return ex2_ftz(__fmul_rn(q, -kHalfLog2e));
 }
-template <> __device__ __forceinline__ float kernel_dF<DARB_GAUSSIAN>(float q, const KernelSpec &) { return -0.5f * __expf(-0.5f * q); }
 
 template <> __device__ __forceinline__ float kernel_F<DARB_HALF_COSINE>(float q, const KernelSpec &) {
     return __cosf(__fmul_rn(q, kPi / 18.0f));
-}
-template <> __device__ __forceinline__ float kernel_dF<DARB_HALF_COSINE>(float q, const KernelSpec &) {
-    return -(kPi / 18.0f) * __sinf(q * (kPi / 18.0f));
 }
 
 template <> __device__ __forceinline__ float kernel_F<DARB_RAISED_COSINE>(float q, const KernelSpec &) {
     return __fmaf_rn(0.5f, __cosf(__fmul_rn(sqrt_newton(q), kPi / 2.5f)), 0.5f);
 }
-template <> __device__ __forceinline__ float kernel_dF<DARB_RAISED_COSINE>(float q, const KernelSpec &) {
+__device__ __forceinline__ float raised_cosine_dF(float q) {
     // -(k/4) sin(k sqrt q) / sqrt q, k = pi/2.5; limit -k^2/4 at q = 0.
     constexpr float k = kPi / 2.5f;
     if (q < 1e-6f) return -0.25f * k * k + (k * k * k * k / 24.0f) * q;
-    const float r = sqrtf(q);
-    return -0.25f * k * __sinf(k * r) / r;
+    return -0.25f * k * __sinf(k * sqrt_newton(q)) * rsqrt_ftz(q);
 }
 
 template <> __device__ __forceinline__ float kernel_F<DARB_MOD_SINC>(float q, const KernelSpec &) {
     // x = pi sqrt(q) / 3, so x^2 = (pi^2 / 9) q; sin(x)/x >= 0 on the main lobe
     return fmaxf(sinc_series(__fmul_rn(q, kPi * kPi / 9.0f)), 0.0f);
 }
-template <> __device__ __forceinline__ float kernel_dF<DARB_MOD_SINC>(float q, const KernelSpec &) {
-    // (x cos x - sin x) / (2 q x), x = pi sqrt(q)/3; series below x = 0.3.
-    const float x = sqrtf(q) * (kPi / 3.0f);
-    if (x < 0.3f) {
-        constexpr float a = kPi * kPi / 9.0f;  // x^2 = a q
-        return -a / 6.0f + (a * a / 60.0f) * q - (a * a * a / 1680.0f) * q * q +
-               (a * a * a * a / 90720.0f) * q * q * q;
-    }
-    float s, c;
-    __sincosf(x, &s, &c);
-    return (x * c - s) / (2.0f * q * x);
-}
 
 template <> __device__ __forceinline__ float kernel_F<DARB_INV_QUADRIC>(float q, const KernelSpec &) {
     return rcp_ftz(__fadd_rn(1.0f, q));
-}
-template <> __device__ __forceinline__ float kernel_dF<DARB_INV_QUADRIC>(float q, const KernelSpec &) {
-    const float r = __fdividef(1.0f, 1.0f + q);
-    return -r * r;
 }
 
 template <> __device__ __forceinline__ float kernel_F<DARB_INV_MULTIQUADRIC>(float q, const KernelSpec &) {
     return rsqrt_ftz(__fadd_rn(1.0f, q));
 }
-template <> __device__ __forceinline__ float kernel_dF<DARB_INV_MULTIQUADRIC>(float q, const KernelSpec &) {
-    const float r = rsqrtf(1.0f + q);
-    return -0.5f * r * r * r;
-}
 
 template <> __device__ __forceinline__ float kernel_F<DARB_PARABOLA>(float q, const KernelSpec &) {
     return __fmaf_rn(q, -1.0f / 9.0f, 1.0f);
 }
-template <> __device__ __forceinline__ float kernel_dF<DARB_PARABOLA>(float, const KernelSpec &) { return -1.0f / 9.0f; }
 
 // The generic member.  u = q / xi exactly when beta = 2, sqrt(q) / xi when beta = 1, else
 // __powf (a few ulp).  The cosines use the hardware approximation on the main lobe and the
@@ -260,11 +233,17 @@ __device__ __forceinline__ float generic_base_du(int base, float u) {
 template <> __device__ __forceinline__ float kernel_F<DARB_GENERIC>(float q, const KernelSpec &ks) {
     return generic_base(ks.base, generic_u(q, ks));
 }
-template <> __device__ __forceinline__ float kernel_dF<DARB_GENERIC>(float q, const KernelSpec &ks) {
-    if (ks.half_beta == 1.0f) return generic_base_du(ks.base, q * ks.inv_xi) * ks.inv_xi;
+// F and dF/dq together, which share u (its power is most of the cost).
+__device__ __forceinline__ void generic_both(float q, const KernelSpec &ks, float &F, float &dF) {
+    const float u = generic_u(q, ks);
+    F = generic_base(ks.base, u);
+    if (ks.half_beta == 1.0f) {
+        dF = generic_base_du(ks.base, u) * ks.inv_xi;
+        return;
+    }
     const float qq = fmaxf(q, 1e-30f);  // one-sided limit at the centre (finite for beta >= 1 on cosines)
-    const float u = generic_u(qq, ks);
-    return generic_base_du(ks.base, u) * ks.half_beta * u / qq;
+    const float uu = q < 1e-30f ? generic_u(qq, ks) : u;
+    dF = generic_base_du(ks.base, uu) * ks.half_beta * __fdividef(uu, qq);
 }
 
 // ---------------------------------------------------------------------------

@@ -12,6 +12,8 @@
 // The support test uses the fixed FP32 sequence conic_q(), and alpha / the kernel value are
 // computed by the same inline code in forward and backward, so the backward re-takes exactly
 // the forward's decisions when it replays a pixel from its last contributor.
+#include <type_traits>
+
 #include "kernels.cuh"
 
 namespace darb {
@@ -23,6 +25,7 @@ struct Bg {
 };
 
 constexpr int kMaxDevicesRender = 64;
+
 
 // The forward's CTA composites a SUB x SUB square of a tile (the squares of a tile walk the same
 // list), PIX pixels a thread.  A warp covers a compact block (LX columns, LY * PIX rows), because it
@@ -51,42 +54,9 @@ template <int TILE> struct FwdOf { using S = FwdShape<TILE, TILE == 8 ? 8 : 16, 
 // its views' lists are short and half the warps then fetch items and records).
 template <int TILE> struct BatchOf { using S = FwdShape<TILE, TILE == 8 ? 8 : 16, TILE == 8 ? 2 : 4>; };
 
-// Resident CTAs per SM the compositing kernels may be compiled for (a register budget);
-// unset, the compiler chooses.  The backward compiles to 64 registers under a budget of 3 or
-// of 4 CTAs per SM (4 stay resident either way), but the schedule it gets for 3 measured
-// 0.186 ms against 0.190 for the half-cosine at 3M / 1080p (Gaussian 0.604 against 0.612).
-#ifndef DARB_BWD_MIN_CTAS
-#define DARB_BWD_MIN_CTAS 3
-#endif
-#ifdef DARB_BWD_MIN_CTAS
-#define DARB_BWD_BOUNDS(nt) __launch_bounds__(nt, DARB_BWD_MIN_CTAS)
-#else
-#define DARB_BWD_BOUNDS(nt) __launch_bounds__(nt)
-#endif
-
-// The backward's shape: with 32-pixel tiles each thread may take more pixels, so that every
-// record read from shared memory and every per-warp reduction serves more pixels.
-#ifndef DARB_BWD_PIX32
-#define DARB_BWD_PIX32 4
-#endif
-template <int TILE>
-struct BwdShape {
-    static constexpr int PIX = TILE == 32 ? DARB_BWD_PIX32 : (TILE == 16 ? 2 : 1);
-    static constexpr int NT = TILE * TILE / PIX;
-    static constexpr int ROWS = TILE / PIX;
-};
-
 // Lane arithmetic on one value or on a pair (the packed two-lane FP32 instructions of sm_100+, which
 // round each lane as the scalar form does).
 template <int L> struct Lanes;
-template <> struct Lanes<1> {
-    using T = float;
-    static __device__ __forceinline__ T dup(float a) { return a; }
-    static __device__ __forceinline__ T mul(T a, T b) { return __fmul_rn(a, b); }
-    static __device__ __forceinline__ T add(T a, T b) { return __fadd_rn(a, b); }
-    static __device__ __forceinline__ T fma(T a, T b, T c) { return __fmaf_rn(a, b, c); }
-    static __device__ __forceinline__ float &at(T &v, int) { return v; }
-};
 template <> struct Lanes<2> {
     using T = float2;
     static __device__ __forceinline__ T dup(float a) { return make_float2(a, a); }
@@ -374,10 +344,38 @@ k_render_fwd_batch(const BatchView *__restrict__ views, int n_views, int total_t
     }
 }
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
+// dF/dq of a pair of values, F the profile there.  Where F gives it, from F; the sinc's from the
+// derivative of its series (to u^7, the next term below 1e-8 on the main lobe), which needs no
+// sine, cosine or division and is nearer the derivative than their quotient was.
+template <int KIND>
+__device__ __forceinline__ float2 kernel_dF2(float2 q, float2 F) {
+    auto dup = [](float a) { return make_float2(a, a); };
+    if constexpr (KIND == DARB_GAUSSIAN) {
+        return __fmul2_rn(F, dup(-0.5f));
+    } else if constexpr (KIND == DARB_HALF_COSINE) {
+        const float2 x = __fmul2_rn(q, dup(kPi / 18.0f));
+        return __fmul2_rn(make_float2(__sinf(x.x), __sinf(x.y)), dup(-(kPi / 18.0f)));
+    } else if constexpr (KIND == DARB_MOD_SINC) {
+        // sum over k of (-1)^k k u^(k - 1) / (2k + 1)!, k = 1 .. 8, times du/dq
+        constexpr float a = kPi * kPi / 9.0f;
+        const float2 u = __fmul2_rn(q, dup(a));
+        float2 r = __ffma2_rn(u, dup(8.0f / 355687428096000.0f), dup(-7.0f / 1307674368000.0f));
+        r = __ffma2_rn(r, u, dup(6.0f / 6227020800.0f));
+        r = __ffma2_rn(r, u, dup(-5.0f / 39916800.0f));
+        r = __ffma2_rn(r, u, dup(4.0f / 362880.0f));
+        r = __ffma2_rn(r, u, dup(-3.0f / 5040.0f));
+        r = __ffma2_rn(r, u, dup(2.0f / 120.0f));
+        r = __ffma2_rn(r, u, dup(-1.0f / 6.0f));
+        return __fmul2_rn(r, dup(a));
+    } else if constexpr (KIND == DARB_INV_QUADRIC) {
+        return __fmul2_rn(F, __fmul2_rn(F, dup(-1.0f)));
+    } else if constexpr (KIND == DARB_INV_MULTIQUADRIC) {
+        return __fmul2_rn(__fmul2_rn(F, F), __fmul2_rn(F, dup(-0.5f)));
+    } else if constexpr (KIND == DARB_PARABOLA) {
+        return dup(-1.0f / 9.0f);
+    } else {
+        return make_float2(raised_cosine_dF(q.x), raised_cosine_dF(q.y));
+    }
 }
 
 // Warp sums of v[0..7] by halving exchanges (4 + 2 + 1 shuffles move half of the remaining
@@ -400,8 +398,33 @@ __device__ __forceinline__ float warp_sum8(const float (&v)[9], int lane, float 
     float c = (b2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, b2 ? b[0] : b[1], 4);
     c += __shfl_xor_sync(0xffffffffu, c, 2);
     c += __shfl_xor_sync(0xffffffffu, c, 1);
-    r8 = warp_sum(v[8]);
+    r8 = v[8];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) r8 += __shfl_xor_sync(0xffffffffu, r8, off);
     return c;  // the sum of v[4 b4 + 2 b3 + b2] = v[lane >> 2]
+}
+
+// Whether the ellipse {q <= qmax} of a record may reach the block of pixel centres [xl, xh] x
+// [yl, yh] (relative to its centre): the least q over the rectangle, which lies on an edge that faces
+// the centre, against qmax with a margin of 5%.  The margin covers the rounding of q, whose
+// relative error grows with the conic's cancellation 1 / (1 - B^2 / (A C)); above 1e4 (or for a
+// conic that is not positive definite in FP32) every record is kept.
+__device__ __forceinline__ bool may_reach(float A, float B, float C, float xl, float xh, float yl, float yh, float qmax) {
+    const float ac = A * C, det = ac - B * B;
+    if (!(det * 1e4f > ac)) return true;
+    const float ex = xl > 0.0f ? xl : xh, ey = yl > 0.0f ? yl : yh;  // the facing edges, where one faces
+    const bool fx = xl > 0.0f || xh < 0.0f, fy = yl > 0.0f || yh < 0.0f;
+    if (!fx && !fy) return true;
+    float m = 3.0e38f;
+    if (fx) {
+        const float dy = fminf(fmaxf(__fdividef(-B * ex, C), yl), yh);
+        m = A * ex * ex + (2.0f * B * ex + C * dy) * dy;
+    }
+    if (fy) {
+        const float dx = fminf(fmaxf(__fdividef(-B * ey, A), xl), xh);
+        m = fminf(m, A * dx * dx + (2.0f * B * dx + C * ey) * ey);
+    }
+    return !(m > 1.05f * qmax);
 }
 
 // Backward: replay each pixel back to front from its last contributor.  With T_k the
@@ -410,159 +433,196 @@ __device__ __forceinline__ float warp_sum8(const float (&v)[9], int lane, float 
 // projection of S on the pixel's upstream gradient g is needed: g . dC/dalpha_k =
 // T_k (g . c_k) - (g . S) / (1 - alpha_k), and g . S grows by (g . c_k) alpha_k T_k per splat,
 // so each pixel carries the scalar g . S instead of three colour channels.
-// Per splat and tile the contributions of a thread's pixels are added in registers, summed
-// over the warp by shuffles, then across warps in shared memory, then added to grad2d with one
-// vector atomic per 4 floats.
-template <int KIND, int TILE>
-__global__ void DARB_BWD_BOUNDS(BwdShape<TILE>::NT)
+//
+// One warp per CTA takes a block of LX x (32 / LX * PIX) pixels, PIX of one column a lane, and walks
+// the tile's run 32 records at a time: each lane gathers one, keeps it if its ellipse may reach
+// the block, and the kept ones are compacted in shared memory.  No barrier beyond the warp and
+// no shared-memory atomics.  The pair body is branch-free (a pair that does not contribute has
+// alpha 0 and leaves T, g . S and every sum as they are) and runs on pairs of pixels with the
+// packed two-lane FP32 instructions.  The gradients w.r.t. centre and conic are sums of s, s dy and
+// s dy^2 over a lane's column (s = dL/dF dF/dq) times powers of the shared dx: three sums a pair
+// instead of five products, with the conic's factors applied once per record.  The warp's nine
+// sums per record leave through vector atomics, a lane per record.
+//
+// Bound by the FP32 and ALU pipes together (two thirds of the issue slots, 50 slots per 32 pairs
+// with the sinc's two series, 88-100 before).  Mod. sinc, 300k splats, 1245 x 825, 16-pixel tiles:
+// 217 us with a CTA per tile, branches per pair and nine products, 127 with eight pixels a lane,
+// 113 with four, 126 with two; half-cosine 100 / 59 / 58 / 75; Gaussian 367 / 228 / 199 / 214; on
+// 32-pixel tiles 273 / 130 / 117 / 130; 8-pixel tiles (8 x 8 blocks, two pixels) 237 -> 118.
+template <int KIND, int LX, int PIX>
+__global__ void __launch_bounds__(32, 24)
 k_render_bwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ values,
              const float2 *__restrict__ mean2d, const float4 *__restrict__ conic_o,
-             const float *__restrict__ rgb, int W, int H, int tiles_x, float qmax, int strict, KernelSpec ks, Bg bg,
-             const float *__restrict__ t_final, const uint32_t *__restrict__ last,
+             const float *__restrict__ rgb, int W, int H, int tiles_x, int tile, float qmax, int strict, KernelSpec ks,
+             Bg bg, const float *__restrict__ t_final, const uint32_t *__restrict__ last,
              const float *__restrict__ dL_dimage, float4 *__restrict__ grad2d) {
     pdl_entry();
-    using S = BwdShape<TILE>;
-    constexpr int NT = S::NT, PIX = S::PIX;
-    constexpr int NW = NT / 32;
-    __shared__ float2 s_xy[NT];
-    __shared__ float4 s_co[NT];
-    __shared__ float s_rgb[NT][3];
-    __shared__ uint32_t s_id[NT];
-    __shared__ float s_acc[NT][9];
-    __shared__ uint32_t s_max[NW];
-
-    const int tile = blockIdx.x;
-    const int tx = tile % tiles_x, ty = tile / tiles_x;
-    const int px = tx * TILE + (threadIdx.x % TILE);
-    const int py0 = ty * TILE + (threadIdx.x / TILE);
+    constexpr int LY = 32 / LX, BH = LY * PIX, NV = PIX / 2;
+    __shared__ float4 s_a[32], s_b[32];            // x, y, A, 2B; C, opacity, red, green
+    __shared__ float s_c[32];                      // blue
+    __shared__ int s_pos[32];
+    __shared__ uint32_t s_id[32];
+    __shared__ float s_sum[32][9];
+    const int lane = threadIdx.x;
+    const int px_parts = tile / LX, parts = px_parts * (tile / BH);
+    const int t = blockIdx.x / parts, part = blockIdx.x % parts;
+    const int x0 = (t % tiles_x) * tile + part % px_parts * LX, y0 = (t / tiles_x) * tile + part / px_parts * BH;
+    const int px = x0 + lane % LX;
     const float fpx = (float)px + 0.5f;
-    const uint2 r = ranges[tile];
-    const int start = (int)r.x;
-    const float qlim = support_limit(qmax, strict);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int start = (int)ranges[t].x;
+    const uint32_t qlim = __float_as_uint(support_limit(qmax, strict));
     const size_t plane = (size_t)W * H;
+    auto dup = [](float a) { return make_float2(a, a); };
 
-    float fpy[PIX], T[PIX], g0[PIX], g1[PIX], g2[PIX], GS[PIX];
-    uint32_t my_last[PIX];
-    uint32_t m = 0;
+    float2 nfpy[NV], T[NV], GS[NV], g0[NV], g1[NV], g2[NV];
+    int my_last[PIX], nlast = 0;
 #pragma unroll
-    for (int k = 0; k < PIX; ++k) {
-        const int py = py0 + k * S::ROWS;
-        fpy[k] = (float)py + 0.5f;
-        T[k] = 1.0f;
-        g0[k] = g1[k] = g2[k] = 0.0f;
-        my_last[k] = 0;
-        if (px < W && py < H) {
-            const size_t pix = (size_t)py * W + px;
-            T[k] = t_final[pix];
-            my_last[k] = last[pix];
-            g0[k] = dL_dimage[pix];
-            g1[k] = dL_dimage[plane + pix];
-            g2[k] = dL_dimage[2 * plane + pix];
-        }
-        GS[k] = T[k] * fmaf(g2[k], bg.b, fmaf(g1[k], bg.g, g0[k] * bg.r));
-        m = max(m, my_last[k]);
-    }
+    for (int v = 0; v < NV; ++v) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if (lane == 0) s_max[warp] = m;
-    for (int i = threadIdx.x; i < NT * 9; i += NT) (&s_acc[0][0])[i] = 0.0f;
-    __syncthreads();
-    int nlast = 0;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) nlast = max(nlast, (int)s_max[w]);
-
-    for (int bend = nlast; bend > 0; bend -= NT) {
-        const int bstart = max(0, bend - NT);
-        const int cnt = bend - bstart;
-        if ((int)threadIdx.x < cnt) {
-            const uint32_t id = values[start + bstart + threadIdx.x];
-            s_id[threadIdx.x] = id;
-            const float2 xy = mean2d[id];
-            float4 co = conic_o[id];
-            co.y = 2.0f * co.y;
-            const float c0 = rgb[3 * (size_t)id], c1 = rgb[3 * (size_t)id + 1], c2 = rgb[3 * (size_t)id + 2];
-            s_xy[threadIdx.x] = xy;
-            s_co[threadIdx.x] = co;
-            s_rgb[threadIdx.x][0] = c0;
-            s_rgb[threadIdx.x][1] = c1;
-            s_rgb[threadIdx.x][2] = c2;
-        }
-        __syncthreads();
-        for (int j = cnt - 1; j >= 0; --j) {
-            const int pos = bstart + j;
-            float v[9];
-#pragma unroll
-            for (int u = 0; u < 9; ++u) v[u] = 0.0f;
-            bool contrib = false;
-            const float2 xy = s_xy[j];
-            const float4 co = s_co[j];
-            const float dx = __fsub_rn(xy.x, fpx);
-#pragma unroll
-            for (int k = 0; k < PIX; ++k) {
-                if (pos >= (int)my_last[k]) continue;
-                const float dy = __fsub_rn(xy.y, fpy[k]);
-                const float q = conic_q(dx, dy, co.x, co.y, co.z);
-                if (!in_support_lim(q, qlim)) continue;
-                const float F = kernel_F<KIND>(q, ks);
-                const float of = __fmul_rn(co.w, F);
-                const float alpha = fminf(kAlphaMax, of);
-                if (alpha < kAlphaMin) continue;
-                contrib = true;
-                const float om = 1.0f - alpha;
-                const float iom = __fdividef(1.0f, om);
-                const float Tk = T[k] * iom;
-                const float c0 = s_rgb[j][0], c1 = s_rgb[j][1], c2 = s_rgb[j][2];
-                const float gc = fmaf(g2[k], c2, fmaf(g1[k], c1, g0[k] * c0));
-                const float dalpha = fmaf(Tk, gc, -GS[k] * iom);
-                const float w = alpha * Tk;
-                GS[k] = fmaf(gc, w, GS[k]);
-                T[k] = Tk;
-                v[6] = fmaf(w, g0[k], v[6]);
-                v[7] = fmaf(w, g1[k], v[7]);
-                v[8] = fmaf(w, g2[k], v[8]);
-                if (!(of > kAlphaMax)) {
-                    v[5] = fmaf(F, dalpha, v[5]);
-                    const float dq = co.w * kernel_dF<KIND>(q, ks) * dalpha;
-                    const float B = 0.5f * co.y;
-                    v[0] = fmaf(2.0f * dq, co.x * dx + B * dy, v[0]);
-                    v[1] = fmaf(2.0f * dq, B * dx + co.z * dy, v[1]);
-                    v[2] = fmaf(dq, dx * dx, v[2]);
-                    v[3] = fmaf(2.0f * dq, dx * dy, v[3]);
-                    v[4] = fmaf(dq, dy * dy, v[4]);
-                }
+        for (int l = 0; l < 2; ++l) {
+            const int py = y0 + lane / LX + (2 * v + l) * LY;
+            float tt = 1.0f, a0 = 0.0f, a1 = 0.0f, a2 = 0.0f;
+            int ml = 0;
+            if (px < W && py < H) {
+                const size_t pix = (size_t)py * W + px;
+                tt = t_final[pix];
+                ml = (int)last[pix];
+                a0 = dL_dimage[pix];
+                a1 = dL_dimage[plane + pix];
+                a2 = dL_dimage[2 * plane + pix];
             }
-            const uint32_t who = __ballot_sync(0xffffffffu, contrib);
-            if (who != 0) {
-                if ((who & (who - 1)) == 0) {  // one contributing lane: it adds its own values
-                    if (contrib) {
+            const float gs = tt * fmaf(a2, bg.b, fmaf(a1, bg.g, a0 * bg.r));
+            (l ? nfpy[v].y : nfpy[v].x) = -((float)py + 0.5f);
+            (l ? T[v].y : T[v].x) = tt;
+            (l ? GS[v].y : GS[v].x) = gs;
+            (l ? g0[v].y : g0[v].x) = a0;
+            (l ? g1[v].y : g1[v].x) = a1;
+            (l ? g2[v].y : g2[v].x) = a2;
+            my_last[2 * v + l] = ml;
+            nlast = max(nlast, ml);
+        }
+    }
+    nlast = (int)__reduce_max_sync(0xffffffffu, (unsigned)nlast);
+    // an upstream gradient that is not finite reaches only the splats that its pixel blended
+    bool odd = false;
 #pragma unroll
-                        for (int u = 0; u < 9; ++u) atomicAdd(&s_acc[j][u], v[u]);
+    for (int v = 0; v < NV; ++v)
+        odd |= !(isfinite(g0[v].x) && isfinite(g0[v].y) && isfinite(g1[v].x) && isfinite(g1[v].y) && isfinite(g2[v].x) &&
+                 isfinite(g2[v].y));
+    odd = __any_sync(0xffffffffu, odd);
+    for (int bend = nlast; bend > 0; bend -= 32) {
+        const int pos = bend - 1 - lane;  // lane 0 the last record: the walk goes back to front
+        bool keep = false;
+        uint32_t id = 0;
+        float2 xy;
+        float4 co;
+        if (pos >= 0) {
+            id = values[start + pos];
+            xy = mean2d[id];
+            co = conic_o[id];
+            keep = may_reach(co.x, co.y, co.z, (float)x0 + 0.5f - xy.x, (float)(x0 + LX) - 0.5f - xy.x,
+                             (float)y0 + 0.5f - xy.y, (float)(y0 + BH) - 0.5f - xy.y, qmax);
+        }
+        const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+        const int n = __popc(kept);
+        if (keep) {
+            const int slot = __popc(kept & ((1u << lane) - 1u));
+            s_a[slot] = make_float4(xy.x, xy.y, co.x, 2.0f * co.y);
+            s_b[slot] = make_float4(co.z, co.w, rgb[3 * (size_t)id], rgb[3 * (size_t)id + 1]);
+            s_c[slot] = rgb[3 * (size_t)id + 2];
+            s_pos[slot] = pos;
+            s_id[slot] = id;
+        }
+        __syncwarp();
+        auto walk = [&](int j, auto masked) {
+            const float4 ra = s_a[j], rb = s_b[j];
+            const float rc = s_c[j];
+            const int rpos = s_pos[j];
+            const float dx1 = __fsub_rn(ra.x, fpx);
+            const float2 dx = dup(dx1), y = dup(ra.y), A = dup(ra.z), B2 = dup(ra.w), Cc = dup(rb.x), o = dup(rb.y);
+            const float2 c0 = dup(rb.z), c1 = dup(rb.w), c2 = dup(rc);
+            float2 S0 = dup(0.0f), S1 = dup(0.0f), S2 = dup(0.0f), SF = dup(0.0f), W0 = dup(0.0f), W1 = dup(0.0f),
+                   W2 = dup(0.0f);
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                const float2 dy = __fadd2_rn(y, nfpy[v]);
+                const float2 e = __ffma2_rn(A, dx, __fmul2_rn(B2, dy));  // conic_q
+                const float2 qr = __ffma2_rn(dx, e, __fmul2_rn(__fmul2_rn(Cc, dy), dy));
+                // outside the support the profile is taken at its limit: finite, so that the pair's zero
+                // weight leaves the sums alone (as unsigned words negative values lie above the limit too)
+                const uint32_t q0 = __float_as_uint(qr.x), q1 = __float_as_uint(qr.y);
+                const float2 q = make_float2(__uint_as_float(min(q0, qlim)), __uint_as_float(min(q1, qlim)));
+                float2 F, dF;
+                if constexpr (KIND == DARB_GENERIC) {  // costly: skipped where no lane is in the support
+                    F = dF = dup(0.0f);
+                    if (__any_sync(0xffffffffu, q0 <= qlim || q1 <= qlim)) {
+                        generic_both(q.x, ks, F.x, dF.x);
+                        generic_both(q.y, ks, F.y, dF.y);
                     }
                 } else {
-                    float r8;
-                    const float r = warp_sum8(v, lane, r8);
-                    if ((lane & 3) == 0) atomicAdd(&s_acc[j][lane >> 2], r);
-                    if (lane == 1) atomicAdd(&s_acc[j][8], r8);
+                    F = kernel_F_lanes<KIND, 2>(q, ks);
+                    dF = kernel_dF2<KIND>(q, F);
                 }
+                const float2 of = __fmul2_rn(o, F);
+                const float al0 = fminf(kAlphaMax, of.x), al1 = fminf(kAlphaMax, of.y);
+                const bool u0 = rpos < my_last[2 * v] && q0 <= qlim && al0 >= kAlphaMin;
+                const bool u1 = rpos < my_last[2 * v + 1] && q1 <= qlim && al1 >= kAlphaMin;
+                const float2 a = make_float2(u0 ? al0 : 0.0f, u1 ? al1 : 0.0f);
+                const float2 om = __ffma2_rn(a, dup(-1.0f), dup(1.0f));
+                const float2 iom = make_float2(rcp_ftz(om.x), rcp_ftz(om.y));
+                const float2 Tk = __fmul2_rn(T[v], iom);
+                float2 h0 = g0[v], h1 = g1[v], h2 = g2[v];
+                if constexpr (decltype(masked)::value) {
+                    if (!u0) h0.x = h1.x = h2.x = 0.0f;
+                    if (!u1) h0.y = h1.y = h2.y = 0.0f;
+                }
+                const float2 gc = __ffma2_rn(h2, c2, __ffma2_rn(h1, c1, __fmul2_rn(h0, c0)));
+                const float2 dal = __ffma2_rn(Tk, gc, __fmul2_rn(__fmul2_rn(GS[v], dup(-1.0f)), iom));
+                const float2 w = __fmul2_rn(a, Tk);
+                GS[v] = __ffma2_rn(gc, w, GS[v]);
+                T[v] = Tk;
+                W0 = __ffma2_rn(w, h0, W0);
+                W1 = __ffma2_rn(w, h1, W1);
+                W2 = __ffma2_rn(w, h2, W2);
+                // the alpha clamp has zero derivative
+                const float2 da = make_float2(u0 && !(of.x > kAlphaMax) ? dal.x : 0.0f,
+                                              u1 && !(of.y > kAlphaMax) ? dal.y : 0.0f);
+                SF = __ffma2_rn(F, da, SF);
+                const float2 sq = __fmul2_rn(dF, da);
+                const float2 p = __fmul2_rn(sq, dy);
+                S0 = __fadd2_rn(S0, sq);
+                S1 = __fadd2_rn(S1, p);
+                S2 = __ffma2_rn(p, dy, S2);
             }
-        }
-        __syncthreads();
-        if ((int)threadIdx.x < cnt) {
-            float *a = s_acc[threadIdx.x];
+            const float t0 = S0.x + S0.y, t1 = S1.x + S1.y, m0 = t0 * dx1;
+            const float sums[9] = {m0, t1, m0 * dx1, t1 * dx1, S2.x + S2.y, SF.x + SF.y, W0.x + W0.y, W1.x + W1.y,
+                                   W2.x + W2.y};
+            float r8;
+            const float r = warp_sum8(sums, lane, r8);
+            if ((lane & 3) == 0) s_sum[j][lane >> 2] = r;
+            if (lane == 1) s_sum[j][8] = r8;
+        };
+        if (odd)
+            for (int j = 0; j < n; ++j) walk(j, std::true_type{});
+        else
+            for (int j = 0; j < n; ++j) walk(j, std::false_type{});
+        __syncwarp();
+        if (lane < n) {
+            const float *s = s_sum[lane];
             bool any = false;
 #pragma unroll
-            for (int u = 0; u < 9; ++u) any |= a[u] != 0.0f;
+            for (int u = 0; u < 9; ++u) any |= s[u] != 0.0f;
             if (any) {
-                float4 *gp = grad2d + 3 * (size_t)s_id[threadIdx.x];
-                atomicAdd(gp, make_float4(a[0], a[1], a[2], a[3]));
-                atomicAdd(gp + 1, make_float4(a[4], a[5], a[6], a[7]));
-                atomicAdd(reinterpret_cast<float *>(gp + 2), a[8]);
+                const float4 ra = s_a[lane], rb = s_b[lane];
+                const float A = ra.z, B = 0.5f * ra.w, C = rb.x, o = rb.y;
+                float4 *gp = grad2d + 3 * (size_t)s_id[lane];
+                atomicAdd(gp, make_float4(2.0f * o * (A * s[0] + B * s[1]), 2.0f * o * (B * s[0] + C * s[1]), o * s[2],
+                                          2.0f * o * s[3]));
+                atomicAdd(gp + 1, make_float4(o * s[4], s[5], s[6], s[7]));
+                atomicAdd(reinterpret_cast<float *>(gp + 2), s[8]);
             }
-#pragma unroll
-            for (int u = 0; u < 9; ++u) a[u] = 0.0f;
         }
-        __syncthreads();
+        __syncwarp();
     }
 }
 
@@ -582,13 +642,14 @@ cudaError_t fwd_t(int n_tiles, const uint2 *ranges, const uint32_t *values, cons
     return cudaGetLastError();
 }
 
-template <int KIND, int TILE>
+template <int KIND, int LX, int PIX>
 cudaError_t bwd_t(int n_tiles, const uint2 *ranges, const uint32_t *values, const float2 *mean2d,
-                  const float4 *conic_o, const float *rgb, const Cam &cam, int tiles_x, float qmax, int strict,
+                  const float4 *conic_o, const float *rgb, const Cam &cam, int tiles_x, int tile, float qmax, int strict,
                   const KernelSpec &ks, const float *t_final, const uint32_t *last, const float *dL, float *grad2d,
                   cudaStream_t st) {
-    launch_k(k_render_bwd<KIND, TILE>, n_tiles, BwdShape<TILE>::NT, 0, st,
-             ranges, values, mean2d, conic_o, rgb, cam.W, cam.H, tiles_x, qmax, strict, ks,
+    const int parts = (tile / LX) * (tile / (32 / LX * PIX));
+    launch_k(k_render_bwd<KIND, LX, PIX>, n_tiles * parts, 32, 0, st,
+             ranges, values, mean2d, conic_o, rgb, cam.W, cam.H, tiles_x, tile, qmax, strict, ks,
              Bg{cam.bg[0], cam.bg[1], cam.bg[2]}, t_final, last, dL, reinterpret_cast<float4 *>(grad2d));
     return cudaGetLastError();
 }
@@ -704,26 +765,16 @@ cudaError_t launch_render_bwd(int kind, int tile, int tiles_x, int tiles_y, cons
     const int n_tiles = tiles_x * tiles_y;
     if (n_tiles == 0) return cudaSuccess;
     const uint2 *rg = reinterpret_cast<const uint2 *>(ranges);
-#define BWD_ARGS (n_tiles, rg, values, mean2d, conic_o, rgb, cam, tiles_x, qmax, strict, ks, t_final, last, dL_dimage, grad2d, st)
-#define BWD_CALL(K, T) bwd_t<K, T> BWD_ARGS
-    if (tile == 8) {
-        switch (kind) {
-        case 0: return BWD_CALL(0, 8); case 1: return BWD_CALL(1, 8); case 2: return BWD_CALL(2, 8);
-        case 3: return BWD_CALL(3, 8); case 4: return BWD_CALL(4, 8); case 5: return BWD_CALL(5, 8);
-        case 6: return BWD_CALL(6, 8); default: return BWD_CALL(7, 8);
-        }
-    } else if (tile == 16) {
-        switch (kind) {
-        case 0: return BWD_CALL(0, 16); case 1: return BWD_CALL(1, 16); case 2: return BWD_CALL(2, 16);
-        case 3: return BWD_CALL(3, 16); case 4: return BWD_CALL(4, 16); case 5: return BWD_CALL(5, 16);
-        case 6: return BWD_CALL(6, 16); default: return BWD_CALL(7, 16);
-        }
-    } else {
-        switch (kind) {
-        case 0: return BWD_CALL(0, 32); case 1: return BWD_CALL(1, 32); case 2: return BWD_CALL(2, 32);
-        case 3: return BWD_CALL(3, 32); case 4: return BWD_CALL(4, 32); case 5: return BWD_CALL(5, 32);
-        case 6: return BWD_CALL(6, 32); default: return BWD_CALL(7, 32);
-        }
+    // 16 x 8 blocks (four pixels a lane), but 16 x 4 where the image has fewer than 26 blocks of 16 x 8 per
+    // SM: the chip is then not full, and a warp's time is its own chain.  Measured (sinc, 300k and 20k
+    // splats): 480 x 270 69 -> 56 us, 640 x 360 63 -> 58 and 54 -> 44, 800 x 450 74 -> 67; at 960 x 540 (27
+    // blocks per SM) 78 either way and 62 -> 59; at 1245 x 825 113 -> 126.
+    const bool few = (long long)n_tiles * (tile * tile / 128) < 26ll * kGridSms;
+#define BWD_ARGS n_tiles, rg, values, mean2d, conic_o, rgb, cam, tiles_x, tile, qmax, strict, ks, t_final, last, dL_dimage, grad2d, st
+#define BWD_CALL(K) (tile == 8 ? bwd_t<K, 8, 2>(BWD_ARGS) : few ? bwd_t<K, 16, 2>(BWD_ARGS) : bwd_t<K, 16, 4>(BWD_ARGS))
+    switch (kind) {
+    case 0: return BWD_CALL(0); case 1: return BWD_CALL(1); case 2: return BWD_CALL(2); case 3: return BWD_CALL(3);
+    case 4: return BWD_CALL(4); case 5: return BWD_CALL(5); case 6: return BWD_CALL(6); default: return BWD_CALL(7);
     }
 #undef BWD_CALL
 #undef BWD_ARGS

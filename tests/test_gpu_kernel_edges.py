@@ -4,9 +4,9 @@ import pytest
 import torch
 
 import oracle
-from paper_2501_12369_gb300 import darb
+from paper_2501_12369_gb300 import darb, synth
 
-from gpu_helpers import to_np
+from gpu_helpers import ambiguity_masked_grad, check_render, gpu_forward, grad_close, to_np
 from test_gpu_density import CFG, RAW, STATE_OF, _case, _device, _t
 
 pytestmark = [pytest.mark.gpu,
@@ -54,3 +54,58 @@ def test_densify_at_block_edges_with_unaligned_moments(n, deg):
             mom = to_np(getattr(so, f"{m}_{STATE_OF[k]}"))
             np.testing.assert_array_equal(mom[:rows], ref_state[f"{m}_{k}"])
             assert np.isnan(mom[rows:]).all()
+
+
+@pytest.mark.parametrize("kernel", ["gaussian", "mod_sinc", "raised_cosine"])
+@pytest.mark.parametrize("tile,width,height", [(32, 992, 511), (32, 1000, 513), (16, 1, 1), (16, 17, 16), (8, 63, 9)])
+def test_compositing_backward_on_either_side_of_its_block_rule(kernel, tile, width, height):
+    """992 x 511 has 3968 blocks of 16 x 8 pixels per 32-pixel tiles (four pixels a lane), 1000 x 513 has 4352;
+    fewer than 3952 take two pixels a lane.  Very small images leave most of a block outside."""
+    s = synth.cluster_scene(1500, seed=31, sh_degree=0)
+    cam = synth.pinhole((0.5, 0.4, 6.0), width, height, 0.8 * max(width, 24), bg=(0.2, 0.1, 0.4))
+    r, sd, proj, bins, img = gpu_forward(s, cam, kernel, tile)
+    ref = oracle.forward(s, cam, kernel, tile=tile)
+    check_render(img, bins, ref, cam, tile)
+    dl = ambiguity_masked_grad(synth.random_image_grad(height, width, seed=4), ref["amb"])
+    _, g2, _ = oracle.gradients(s, cam, dl, kernel, tile=tile)
+    got = darb.darb_render_bwd(proj, s.n, bins, cam, r.kparams, tile, img, _t(dl.astype(np.float32)))
+    torch.cuda.synchronize()
+    for u in range(9):
+        grad_close(f"grad2d[{u}]", to_np(got)[:, u], np.asarray(g2)[:, u])
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_gradient_that_is_not_finite_stays_with_the_splats_its_pixel_blended(bad):
+    s = synth.cluster_scene(4000, seed=8, sh_degree=0)
+    cam = synth.fibonacci_cameras(16, 6.0, 150, 97, 120.0)[2]
+    r, sd, proj, bins, img = gpu_forward(s, cam, "half_cosine", 16)
+    dl = synth.random_image_grad(97, 150, seed=4)
+    clean = to_np(darb.darb_render_bwd(proj, s.n, bins, cam, r.kparams, 16, img, _t(dl)))
+    y, x = 50, 75
+    one = np.zeros_like(dl)
+    one[:, y, x] = 1.0
+    touched = (to_np(darb.darb_render_bwd(proj, s.n, bins, cam, r.kparams, 16, img, _t(one)))[:, 6:9] != 0).any(axis=1)
+    dl[1, y, x] = bad
+    got = to_np(darb.darb_render_bwd(proj, s.n, bins, cam, r.kparams, 16, img, _t(dl)))
+    assert 0 < touched.sum() < s.n
+    assert not np.isfinite(got[touched]).all(axis=1).any()
+    assert np.isfinite(got[~touched]).all()
+    np.testing.assert_allclose(got[~touched], clean[~touched], rtol=1e-4, atol=1e-5 * np.abs(clean).max())
+
+
+@pytest.mark.parametrize("kernel", oracle.KERNEL_NAMES)
+def test_conic_that_rounds_to_indefinite_adds_nothing_outside_its_support(kernel):
+    """A record whose conic is not positive definite in FP32 has q far below 0 (where the Gaussian overflows)
+    and far above its limit (where the sinc's series does): such pairs carry weight 0 and every gradient
+    stays finite and as it is without the record."""
+    s = synth.cluster_scene(500, seed=3, sh_degree=0)
+    cam = synth.pinhole((0.0, 0.0, 6.0), 64, 48, 60.0)
+    r, sd, proj, bins, img = gpu_forward(s, cam, kernel, 16)
+    lists, ranges = to_np(bins.values), to_np(bins.ranges)
+    first = np.unique([lists[a] for a, b in ranges if b > a])  # the nearest record of every tile
+    proj.conic_o[torch.from_numpy(first.astype(np.int64)).cuda()] = torch.tensor([1e6, 3e6, 1e6, 0.5], device="cuda")
+    proj.mean2d[torch.from_numpy(first.astype(np.int64)).cuda()] += 1000.25
+    img = darb.darb_render_fwd(proj, bins, cam, r.kparams, 16)
+    assert torch.isfinite(img.image).all()
+    g = to_np(darb.darb_render_bwd(proj, s.n, bins, cam, r.kparams, 16, img, _t(synth.random_image_grad(48, 64, seed=4))))
+    assert np.isfinite(g).all() and (g[first] == 0).all() and np.abs(g).max() > 0
