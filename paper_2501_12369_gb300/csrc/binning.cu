@@ -39,6 +39,7 @@
 // timeout the status word is set and successors are released), and staging in shared memory so
 // the scatter leaves in digit runs.
 #include <algorithm>
+#include <cooperative_groups.h>
 #include <mutex>
 #include <utility>
 
@@ -1474,6 +1475,202 @@ k_keys64(const uint32_t *__restrict__ ranges, const uint32_t *__restrict__ vals,
     }
 }
 
+// ---------------------------------------------------------------------------- small scenes
+//
+// The whole depth order of a small scene in one launch: the depth keys, four stable 8-bit LSD
+// passes, and the instance offsets, partition owners and M in depth order, by one cluster of up to
+// 8 CTAs.  The keys live in the CTAs' shared memory, position p in CTA p / S at p % S; a pass ranks
+// its CTA's keys as k_onesweep does, exchanges the digit counts through distributed shared memory
+// and stores the keys in digit runs into the CTAs of their new positions, with two cluster barriers
+// and no look-back.  Culled splats carry the all-ones key and sort behind the visible ones.
+// Bound by latency (barriers and the ranking's votes).  It replaces seven launches (compaction,
+// digit scan, four passes of one to a few CTAs, offsets: 59 us at 1000 splats, 70 at 20000) by one
+// of 19 and 36 us; darb_bin_sort, 1080p, 16-pixel tiles, at 1000 / 5000 / 16000 / 30000 splats:
+// 61 / 64 / 68 / 72 -> 52 / 52 / 54 / 64 us.  At 65000 (eight items a thread) it took 96 against 80.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallMaxItems = 4, kSmallMaxCtas = 8;
+constexpr int kSmallMax = kSmallThreads * kSmallMaxItems * kSmallMaxCtas;  // 32768 splats
+
+template <int ITEMS>
+struct SmallSmem {
+    static constexpr int S = kSmallThreads * ITEMS;  // positions per CTA
+    uint32_t key[S], val[S];    // the CTA's positions, written by the whole cluster
+    uint32_t skey[S], sval[S];  // its keys of a pass, sorted by the digit, so that they leave in runs
+    uint32_t wh[kSmallThreads / 32][256];  // per-warp digit counts, then their offsets within the CTA's digit
+    uint32_t total[256];                   // the CTA's count of every digit (read by the whole cluster)
+    uint32_t excl[256], base[256];         // where they start in the CTA's sorted keys, and among all
+    unsigned long long warp[kSmallThreads / 32 + 1];
+    unsigned long long sum;  // the CTA's instances (read by the whole cluster)
+};
+
+template <int ITEMS>
+__global__ void __launch_bounds__(kSmallThreads)
+k_small_depth_sort(int n, const int *__restrict__ radius, const float *__restrict__ depth,
+                   const uint32_t *__restrict__ tiles, uint32_t *__restrict__ order, uint32_t *__restrict__ num,
+                   uint32_t *status, unsigned long long capacity, uint32_t *__restrict__ offs,
+                   uint2 *__restrict__ bounds, uint32_t max_parts) {
+    pdl_entry();
+    extern __shared__ __align__(16) unsigned char smem[];
+    using Smem = SmallSmem<ITEMS>;
+    Smem &sm = *reinterpret_cast<Smem *>(smem);
+    constexpr uint32_t S = Smem::S;
+    constexpr int NW = kSmallThreads / 32;
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const uint32_t rank = cluster.block_rank(), ctas = cluster.num_blocks();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t first = rank * S, lt = lanemask_lt();
+    // item `it` of a lane is position warp * 32 * ITEMS + it * 32 + lane of the CTA (stable ranks)
+    const uint32_t slot0 = (uint32_t)(warp * 32 * ITEMS + lane);
+    uint32_t k[ITEMS], v[ITEMS], rk[ITEMS];
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        const uint32_t i = first + slot0 + it * 32;
+        v[it] = i;
+        k[it] = 0xffffffffu;  // culled splats, and positions past n
+        if (i < (uint32_t)n && radius[i] != 0) k[it] = __float_as_uint(depth[i]);
+    }
+#pragma unroll 1
+    for (int shift = 0; shift < 32; shift += 8) {
+        for (int i = tid; i < NW * 256; i += kSmallThreads) (&sm.wh[0][0])[i] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            const uint32_t d = (k[it] >> shift) & 255u;
+            const uint32_t peers = match_digit(d, 8);
+            const int leader = __ffs(peers) - 1;
+            uint32_t old = 0;
+            if (lane == leader) old = atomicAdd(&sm.wh[warp][d], (uint32_t)__popc(peers));
+            rk[it] = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lt);
+        }
+        __syncthreads();
+        {  // four neighbouring lanes per digit, eight warps' counts each
+            const int d = tid >> 2, w0 = (tid & 3) * (NW / 4);
+            uint32_t c[NW / 4], mine = 0;
+#pragma unroll
+            for (int w = 0; w < NW / 4; ++w) {
+                c[w] = sm.wh[w0 + w][d];
+                mine += c[w];
+            }
+            uint32_t incl = mine;
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o, 4);
+                if ((tid & 3) >= o) incl += y;
+            }
+            uint32_t run = incl - mine;
+#pragma unroll
+            for (int w = 0; w < NW / 4; ++w) {
+                sm.wh[w0 + w][d] = run;
+                run += c[w];
+            }
+            if ((tid & 3) == 3) sm.total[d] = incl;
+        }
+        cluster.sync();  // the counts of every CTA; and every CTA holds its keys in registers
+        uint32_t before = 0, all = 0, own = 0;
+        if (tid < 256) {
+            own = sm.total[tid];
+            uint32_t x[kSmallMaxCtas];  // every CTA's count in flight at once
+#pragma unroll
+            for (uint32_t c = 0; c < kSmallMaxCtas; ++c)
+                x[c] = c >= ctas ? 0u : c == rank ? own : cluster.map_shared_rank(sm.total, c)[tid];
+#pragma unroll
+            for (uint32_t c = 0; c < kSmallMaxCtas; ++c) {
+                all += x[c];
+                before += c < rank ? x[c] : 0u;
+            }
+        }
+        unsigned long long sum;  // both scans at once: all CTAs' counts above, the CTA's own below
+        const unsigned long long ex =
+            block_exclusive_scan<kSmallThreads>((unsigned long long)all << 32 | own, sm.warp, sum);
+        if (tid < 256) {
+            sm.excl[tid] = (uint32_t)ex;
+            sm.base[tid] = (uint32_t)(ex >> 32) + before;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            const uint32_t d = (k[it] >> shift) & 255u;
+            const uint32_t pos = sm.excl[d] + sm.wh[warp][d] + rk[it];
+            sm.skey[pos] = k[it];
+            sm.sval[pos] = v[it];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            const uint32_t j = (uint32_t)(it * kSmallThreads + tid), kk = sm.skey[j], d = (kk >> shift) & 255u;
+            const uint32_t dst = sm.base[d] + (j - sm.excl[d]);
+            cluster.map_shared_rank(sm.key, dst / S)[dst % S] = kk;
+            cluster.map_shared_rank(sm.val, dst / S)[dst % S] = sm.sval[j];
+        }
+        cluster.sync();  // every key has arrived; the counts may be cleared
+        if (shift < 24) {
+#pragma unroll
+            for (int it = 0; it < ITEMS; ++it) {
+                k[it] = sm.key[slot0 + it * 32];
+                v[it] = sm.val[slot0 + it * 32];
+            }
+        }
+    }
+    // instance offsets in depth order; a thread takes ITEMS consecutive positions
+    uint32_t cnt[ITEMS];
+    unsigned long long mine = 0;
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t p = (uint32_t)(tid * ITEMS + j), id = sm.val[p];
+        cnt[j] = 0;
+        if (first + p < (uint32_t)n) {
+            order[first + p] = id;
+            if (sm.key[p] != 0xffffffffu) cnt[j] = tiles[id];
+        }
+        mine += cnt[j];
+    }
+    unsigned long long total;
+    const unsigned long long ex = block_exclusive_scan<kSmallThreads>(mine, sm.warp, total);
+    if (tid == 0) sm.sum = total;
+    cluster.sync();
+    unsigned long long g = 0, M = 0;
+    unsigned long long sums[kSmallMaxCtas];
+#pragma unroll
+    for (uint32_t c = 0; c < kSmallMaxCtas; ++c) sums[c] = c < ctas ? *cluster.map_shared_rank(&sm.sum, c) : 0ull;
+#pragma unroll
+    for (uint32_t c = 0; c < kSmallMaxCtas; ++c) {
+        M += sums[c];
+        g += c < rank ? sums[c] : 0ull;
+    }
+    cluster.sync();  // no CTA leaves while its sum is being read
+    if (rank == 0 && tid == 0) {
+        *num = M > 0xffffffffull ? 0xffffffffu : (uint32_t)M;
+        if (M > capacity) atomicExch(status, (uint32_t)DARB_ERR_CAPACITY);
+        offs[n] = (uint32_t)M;
+    }
+    constexpr uint32_t T = kSortTile;
+    uint32_t o0 = (uint32_t)(g + ex);
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t p = first + (uint32_t)(tid * ITEMS + j), o1 = o0 + cnt[j];
+        if (p < (uint32_t)n) offs[p] = o0;
+        if (cnt[j]) {  // the partitions whose first or last instance this position owns
+            for (uint32_t q = (o0 + T - 1) / T; q < (o1 + T - 1) / T && q < max_parts; ++q) bounds[q].x = p;
+            for (uint32_t q = (o0 + 1 + T - 1) / T - 1; q + 1 <= o1 / T && q < max_parts; ++q) bounds[q].y = p;
+            if (o1 == (uint32_t)M && (o1 - 1) / T < max_parts) bounds[(o1 - 1) / T].y = p;
+        }
+        o0 = o1;
+    }
+}
+
+template <int ITEMS>
+cudaError_t launch_small(int n, const ProjectedIn &proj, uint32_t *order, const BinOut &out, unsigned long long cap,
+                         uint32_t *offs, uint2 *bounds, uint32_t max_parts, cudaStream_t st) {
+    const size_t smem = sizeof(SmallSmem<ITEMS>);
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_small_depth_sort<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int ctas = (n + SmallSmem<ITEMS>::S - 1) / SmallSmem<ITEMS>::S;
+    launch_cluster(k_small_depth_sort<ITEMS>, ctas, ctas, kSmallThreads, smem, st, n, proj.radius, proj.depth,
+                   proj.tiles_touched, order, out.num_instances, out.status, cap, offs, bounds, max_parts);
+    return cudaGetLastError();
+}
+
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 PassSpec split_bits(int total_bits) {
@@ -1698,6 +1895,11 @@ struct SideJoin {
 };
 }  // namespace
 
+// The depth order of at most kSmallMax splats by one cluster (1), or by the passes of any size (0).
+#ifndef DARB_SMALL_SORT
+#define DARB_SMALL_SORT 1
+#endif
+
 // Per-tile counts beside the depth passes (1), or in line on the caller's stream (0).
 #ifndef DARB_TILE_COUNTS_FORK
 #define DARB_TILE_COUNTS_FORK 1
@@ -1811,7 +2013,39 @@ cudaError_t launch_bin_sort(int n, const ProjectedIn &proj, int tiles_x, int til
     const uint32_t *order = nullptr;  // sorted splat ids
     const uint32_t *n_vis_dev = nullptr;  // visible count, when order starts with exactly the visible splats
     uint32_t *sums = reinterpret_cast<uint32_t *>(at(17));
-    if (n > 0) {
+    uint32_t *offs = reinterpret_cast<uint32_t *>(at(15));
+    uint2 *bounds = kPassOnesweep ? reinterpret_cast<uint2 *>(at(20)) : nullptr;
+    const uint32_t max_parts = (uint32_t)((capacity + kSortTile - 1) / kSortTile);
+    const bool small = kPassOnesweep && DARB_SMALL_SORT && n > 0 && n <= kSmallMax;
+    auto fork_tile_counts = [&](const uint32_t *ids, const uint32_t *count) {
+        // the per-tile counts need no depth order: they walk the splats in index order (coalesced
+        // reads), and on the side stream they run beside the (latency-bound) depth order
+        cudaStream_t ts = st;
+        if (side) {
+            TRY(cudaEventRecord(side->fork, st));
+            TRY(cudaStreamWaitEvent(side->s, side->fork, 0));
+            ts = side->s;
+        }
+        TRY(launch_tile_counts(n, ids, count, proj, sc, rt, tiles_x, tiles_y, diff, counts, out, cap, tps, tbase, ts));
+        if (side) {
+            TRY(cudaEventRecord(side->join, side->s));
+            side_join.st = st;
+            side_join.ev = side->join;
+            side_join.pending = true;
+        }
+        tile_counts_done = true;
+        return cudaSuccess;
+    };
+    if (small) {
+        TRY(fork_tile_counts(nullptr, nullptr));
+        // two positions a thread up to 16384 splats, four to 32768: the fewer, the shorter a pass
+        uint32_t *o = vbuf[1];
+        order = o;
+        if (n <= kSmallThreads * 2 * kSmallMaxCtas)
+            TRY(launch_small<2>(n, proj, o, out, cap, offs, bounds, max_parts, st));
+        else
+            TRY(launch_small<4>(n, proj, o, out, cap, offs, bounds, max_parts, st));
+    } else if (n > 0) {
         const PassSpec dps = split_bits(32);
         uint32_t *dph = reinterpret_cast<uint32_t *>(at(12));
         uint32_t *dbase = reinterpret_cast<uint32_t *>(at(9));
@@ -1834,26 +2068,7 @@ cudaError_t launch_bin_sort(int n, const ProjectedIn &proj, int tiles_x, int til
             n_vis_dev = nv;
             vin = vbuf[0];
             launch_k(k_hist_scan, dps.passes, 256, 0, st, dhist, dbase);
-            if (kTileCountsEarly) {
-                // the per-tile counts need no depth order: walk the visible splats in index order
-                // (coalesced reads) before the depth passes overwrite this compacted list; on the
-                // side stream they run beside the (latency-bound) depth passes
-                cudaStream_t ts = st;
-                if (side) {
-                    TRY(cudaEventRecord(side->fork, st));
-                    TRY(cudaStreamWaitEvent(side->s, side->fork, 0));
-                    ts = side->s;
-                }
-                TRY(launch_tile_counts(n, vbuf[0], nv, proj, sc, rt, tiles_x, tiles_y, diff, counts, out, cap, tps,
-                                       tbase, ts));
-                if (side) {
-                    TRY(cudaEventRecord(side->join, side->s));
-                    side_join.st = st;
-                    side_join.ev = side->join;
-                    side_join.pending = true;
-                }
-                tile_counts_done = true;
-            }
+            if (kTileCountsEarly) TRY(fork_tile_counts(vbuf[0], nv));
         } else {
             launch_k(k_depth_keys, (n + 255) / 256, 256, 0, st, n, proj.radius, proj.depth, kbuf[0]);
         }
@@ -1890,11 +2105,9 @@ cudaError_t launch_bin_sort(int n, const ProjectedIn &proj, int tiles_x, int til
         order = vin;
     }
     // 2) scan of tiles_touched in depth order (with the onesweep passes: chained, in step 4)
-    uint32_t *offs = reinterpret_cast<uint32_t *>(at(15));
-    uint2 *bounds = kPassOnesweep ? reinterpret_cast<uint2 *>(at(20)) : nullptr;
-    const uint32_t max_parts = (uint32_t)((capacity + kSortTile - 1) / kSortTile);
-    const bool chained = DARB_CHAINED_SCANS && kPassOnesweep && n_vis_dev;
-    if (chained) {
+    const bool chained = small || (DARB_CHAINED_SCANS && kPassOnesweep && n_vis_dev);
+    if (small) {  // offsets, owners and M came with the depth order
+    } else if (chained) {
         // 4, ahead) per-position offsets and owners, M and the capacity check in one chained pass
         if (nb > 0)
             launch_k(k_splat_offsets_chained, nb, kScanThreads, 0, st, n, order, proj.tiles_touched, n_vis_dev,

@@ -6,7 +6,7 @@ import torch
 import oracle
 from paper_2501_12369_gb300 import darb, synth
 
-from gpu_helpers import ambiguity_masked_grad, check_render, gpu_forward, grad_close, to_np
+from gpu_helpers import ambiguity_masked_grad, check_lists, check_render, gpu_forward, grad_close, to_np
 from test_gpu_density import CFG, RAW, STATE_OF, _case, _device, _t
 
 pytestmark = [pytest.mark.gpu,
@@ -109,3 +109,23 @@ def test_conic_that_rounds_to_indefinite_adds_nothing_outside_its_support(kernel
     assert torch.isfinite(img.image).all()
     g = to_np(darb.darb_render_bwd(proj, s.n, bins, cam, r.kparams, 16, img, _t(synth.random_image_grad(48, 64, seed=4))))
     assert np.isfinite(g).all() and (g[first] == 0).all() and np.abs(g).max() > 0
+
+
+@pytest.mark.parametrize("n", [1, 31, 1025, 2048, 2049, 16384, 16385, 32768, 32769])
+def test_depth_order_of_small_scenes_at_the_edges_of_its_cluster(n):
+    """2048 positions a CTA and up to 8 CTAs to 16384 splats, 4096 to 32768, the passes of any size beyond; with equal depths (which keep splat order) and culled splats."""
+    s = synth.cluster_scene(n, seed=n, sh_degree=0)
+    s.means[::7] = s.means[0]
+    s.means[3::11, :] *= np.float32(40.0)  # outside the frame or behind the camera
+    cam = synth.fibonacci_cameras(16, 6.0, 205, 121, 160.0)[5]
+    r, sd, proj, bins, img = gpu_forward(s, cam, "half_cosine", 16)
+    ref = oracle.project(s, cam, oracle.kernel_params("half_cosine"), 16, True)
+    lists = oracle.build_lists(ref, cam, 16)
+    check_lists(bins, lists)
+    if lists["M"] > 1:  # one instance too many, found on the device
+        cap = lists["M"] - 1
+        ws = torch.empty(darb.darb_bin_sort_workspace_size(n, 16, cam, cap), dtype=torch.uint8, device="cuda")
+        b = darb.darb_bin_sort(proj, n, 16, cam, ws, cap, sync=False)
+        torch.cuda.synchronize()
+        assert int(to_np(b.status)[0]) == 3 and int(to_np(b.num_instances)[0]) == lists["M"]
+        assert (to_np(b.ranges) == 0).all()
