@@ -219,8 +219,8 @@ darb_status darb_bin_sort_workspace_size(int32_t n, int32_t tile, const darb_cam
  * the per-tile ranges, [0, 0) for a tile without instances.  strategy: a darb_sort_strategy.
  * proj: darb_preprocess outputs.  workspace: device, at least
  * darb_bin_sort_workspace_size bytes, contents scratch.  capacity: entries of
- * out->keys / out->values (< 2^30).  num_instances_host: if non-NULL the call
- * synchronises the stream once to read M and returns DARB_ERR_CAPACITY when
+ * out->keys / out->values (< 2^30).  num_instances_host: if non-NULL the call waits
+ * once, until the stream has counted M, to read it and returns DARB_ERR_CAPACITY when
  * M > capacity (outputs then undefined); if NULL nothing synchronises, the sort is
  * sized by capacity, and an overflow is reported in out->status with every tile range
  * left empty (so a following darb_render_fwd draws only the background).  The per-tile counts
