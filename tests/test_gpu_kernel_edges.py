@@ -129,3 +129,15 @@ def test_depth_order_of_small_scenes_at_the_edges_of_its_cluster(n):
         torch.cuda.synchronize()
         assert int(to_np(b.status)[0]) == 3 and int(to_np(b.num_instances)[0]) == lists["M"]
         assert (to_np(b.ranges) == 0).all()
+
+
+@pytest.mark.parametrize("width,height", [(5, 3), (31, 33), (32, 32), (33, 65), (1300, 700)])
+def test_dssim_at_tile_edges(width, height):
+    """Images smaller than a halo, one tile, just over it, and (1300 x 700) more tiles than the backward has CTAs."""
+    img, tgt = synth.random_target(height, width, seed=5), synth.random_target(height, width, seed=6)
+    img[:, ::2] = tgt[:, ::2]
+    dl, loss = darb.darb_l1_dssim_loss(_t(img), _t(tgt), 0.2)
+    ref_loss, ref_dl, ref_ssim = oracle.l1_dssim_loss(img, tgt, 0.2)
+    torch.cuda.synchronize()
+    assert abs(float(loss[0]) - ref_loss) <= 2e-6 and abs(float(loss[1]) - ref_ssim) <= 4e-6
+    grad_close("dL", to_np(dl), ref_dl)
