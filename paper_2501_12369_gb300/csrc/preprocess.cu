@@ -123,24 +123,6 @@ __device__ __forceinline__ void load_sh(const float *__restrict__ sh, int i, flo
     }
 }
 
-template <int DEG>
-__device__ __forceinline__ void store_sh(float *__restrict__ dsh, int i, const float (*c)[3]) {
-    constexpr int K = (DEG + 1) * (DEG + 1);
-    if constexpr ((K * 3) % 4 == 0) {
-        float4 *p = reinterpret_cast<float4 *>(dsh + (size_t)i * K * 3);
-        float buf[K * 3];
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-            for (int ch = 0; ch < 3; ++ch) buf[3 * k + ch] = c[k][ch];
-#pragma unroll
-        for (int j = 0; j < K * 3 / 4; ++j) p[j] = make_float4(buf[4 * j], buf[4 * j + 1], buf[4 * j + 2], buf[4 * j + 3]);
-    } else {
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-            for (int ch = 0; ch < 3; ++ch) dsh[((size_t)i * K + k) * 3 + ch] = c[k][ch];
-    }
-}
-
 // The fixed FP32 projection sequence.  Returns false when the splat is culled.
 struct Geom {
     float t[3];
@@ -593,33 +575,6 @@ __device__ __forceinline__ void splat_backward(int i, const float *__restrict__ 
 }
 
 
-template <int DEG>
-__global__ void __launch_bounds__(256)
-k_preprocess_bwd(int n, const float *__restrict__ means, const float *__restrict__ scales,
-                 const float4 *__restrict__ quats, const float *__restrict__ sh, Cam cam, float psi,
-                 const int *__restrict__ radius, const uint8_t *__restrict__ clamped,
-                 const float4 *__restrict__ grad2d, GradOut out) {
-    pdl_entry();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    constexpr int K = (DEG + 1) * (DEG + 1);
-    float dm[3] = {0.f, 0.f, 0.f}, ds[3] = {0.f, 0.f, 0.f}, dq[4] = {0.f, 0.f, 0.f, 0.f}, dop = 0.f;
-    float dcoef[K][3];
-#pragma unroll
-    for (int k = 0; k < K; ++k) dcoef[k][0] = dcoef[k][1] = dcoef[k][2] = 0.0f;
-    if (radius[i] != 0)
-        splat_backward<DEG>(
-            i, means, scales, quats, [&](float(*c)[3]) { load_sh<DEG>(sh, i, c); }, cam, psi, clamped[i], grad2d, dm,
-            ds, dq, dop, dcoef);
-    for (int j = 0; j < 3; ++j) {
-        out.dmeans[3 * (size_t)i + j] = dm[j];
-        out.dscales[3 * (size_t)i + j] = ds[j];
-    }
-    reinterpret_cast<float4 *>(out.dquats)[i] = make_float4(dq[0], dq[1], dq[2], dq[3]);
-    out.dopacities[i] = dop;
-    store_sh<DEG>(out.dsh, i, dcoef);
-}
-
 // The same gradients applied at once by Adam to the raw parameters (log-scales, opacity
 // logits), refreshing the activated copies; no gradient goes through HBM.
 //
@@ -638,7 +593,92 @@ struct BwdAdamStage {
     static constexpr int PAD = (ROW % 4 == 0 && (ROW / 4) % 2 == 0) ? ROW + 4 : ROW;
 };
 
+// One splat's SH gradients into its row of the block's segment.
+template <int DEG>
+__device__ __forceinline__ void stage_sh_row(float *row, const float *dc) {
+    constexpr int ROW = BwdAdamStage<DEG>::ROW;
+    if constexpr (ROW % 4 == 0) {
+#pragma unroll
+        for (int u = 0; u < ROW / 4; ++u)
+            *reinterpret_cast<float4 *>(row + 4 * u) = make_float4(dc[4 * u], dc[4 * u + 1], dc[4 * u + 2], dc[4 * u + 3]);
+    } else {
+#pragma unroll
+        for (int u = 0; u < ROW; ++u) row[u] = dc[u];
+    }
+}
+
 constexpr int kBwdAdamThreads = 128;
+
+// A block's rows of one gradient: count floats from shared memory (float4 j of the segment by
+// grad4(j)) to consecutive addresses, 16 bytes a lane where dst is aligned.
+template <class Grad4>
+__device__ __forceinline__ void block_store(int count, float *__restrict__ dst, Grad4 grad4) {
+    const bool vec = (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
+    for (int j = threadIdx.x; 4 * j < count; j += kBwdAdamThreads) {
+        const float4 g = grad4(j);
+        if (vec && 4 * j + 4 <= count) {
+            reinterpret_cast<float4 *>(dst)[j] = g;
+        } else {
+            const float gs[4] = {g.x, g.y, g.z, g.w};
+            for (int u = 0; u < 4 && 4 * j + u < count; ++u) dst[4 * j + u] = gs[u];
+        }
+    }
+}
+
+// The gradients as arrays (the unfused step).  HBM-bound: phase 1 of the fused kernel below, then
+// every gradient leaves the block as one contiguous range.  With each thread storing its own rows
+// the 192-byte SH rows and the 12-byte ones left the warps in scattered pieces: 95 -> 77 us (1M splats,
+// degree 3).  Degree 0 has no long rows and stores directly (staged 117 us against 111 with Adam).
+template <int DEG>
+__global__ void __launch_bounds__(kBwdAdamThreads, DEG == 2 ? 4 : 6)
+k_preprocess_bwd(int n, const float *__restrict__ means, const float *__restrict__ scales,
+                 const float4 *__restrict__ quats, const float *__restrict__ sh, Cam cam, float psi,
+                 const int *__restrict__ radius, const uint8_t *__restrict__ clamped,
+                 const float4 *__restrict__ grad2d, GradOut out) {
+    pdl_entry();
+    using S = BwdAdamStage<DEG>;
+    constexpr int K = S::K, ROW = S::ROW, PAD = S::PAD, NT = kBwdAdamThreads;
+    constexpr bool STAGED = DEG >= 1;
+    __shared__ __align__(16) float s_means[STAGED ? NT * 3 : 4];
+    __shared__ __align__(16) float s_scales[STAGED ? NT * 3 : 4];
+    __shared__ __align__(16) float s_opac[STAGED ? NT : 4];
+    __shared__ __align__(16) float s_sh[STAGED ? NT * PAD : 4];
+    const int t = threadIdx.x, i0 = blockIdx.x * NT, i = i0 + t, cnt = min(NT, n - i0);
+    if (i < n) {
+        float dm[3] = {0.f, 0.f, 0.f}, ds[3] = {0.f, 0.f, 0.f}, dq[4] = {0.f, 0.f, 0.f, 0.f}, dop = 0.f;
+        float dcoef[K][3];
+#pragma unroll
+        for (int k = 0; k < K; ++k) dcoef[k][0] = dcoef[k][1] = dcoef[k][2] = 0.0f;
+        if (radius[i] != 0)
+            splat_backward<DEG>(
+                i, means, scales, quats, [&](float(*c)[3]) { load_sh<DEG>(sh, i, c); }, cam, psi, clamped[i], grad2d, dm,
+                ds, dq, dop, dcoef);
+        reinterpret_cast<float4 *>(out.dquats)[i] = make_float4(dq[0], dq[1], dq[2], dq[3]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            (STAGED ? s_means[3 * t + j] : out.dmeans[3 * (size_t)i + j]) = dm[j];
+            (STAGED ? s_scales[3 * t + j] : out.dscales[3 * (size_t)i + j]) = ds[j];
+        }
+        (STAGED ? s_opac[t] : out.dopacities[i]) = dop;
+        if constexpr (STAGED) {
+            stage_sh_row<DEG>(&s_sh[t * PAD], &dcoef[0][0]);
+        } else {
+#pragma unroll
+            for (int ch = 0; ch < 3; ++ch) out.dsh[3 * (size_t)i + ch] = dcoef[0][ch];
+        }
+    }
+    if constexpr (!STAGED) return;
+    __syncthreads();
+    auto flat = [](const float *s) { return [s](int j) { return reinterpret_cast<const float4 *>(s)[j]; }; };
+    block_store(ROW * cnt, out.dsh + (size_t)i0 * ROW, [&](int j) {
+        if constexpr (PAD == ROW) return reinterpret_cast<const float4 *>(s_sh)[j];
+        const int r = j / (ROW / 4 > 0 ? ROW / 4 : 1), col = 4 * (j - r * (ROW / 4));
+        return *reinterpret_cast<const float4 *>(&s_sh[r * PAD + col]);
+    });
+    block_store(3 * cnt, out.dmeans + 3 * (size_t)i0, flat(s_means));
+    block_store(3 * cnt, out.dscales + 3 * (size_t)i0, flat(s_scales));
+    block_store(cnt, out.dopacities + i0, flat(s_opac));
+}
 
 // float4s in flight per thread and array in the Adam walk, and whether its parameter / moment
 // traffic uses the streaming (evict-first) cache hints.
@@ -760,16 +800,7 @@ k_preprocess_bwd_adam(int n, darb_train_params P, darb_adam_state A, AdamConsts 
         *reinterpret_cast<float4 *>(&s_quat[4 * t]) = make_float4(dq[0], dq[1], dq[2], dq[3]);
         const float o = P.opacities[i];
         s_logit[t] = dop * (o * (1.0f - o));
-        const float *dc = &dcoef[0][0];
-        if constexpr (ROW % 4 == 0) {
-#pragma unroll
-            for (int u = 0; u < ROW / 4; ++u)
-                *reinterpret_cast<float4 *>(&s_sh[t * PAD + 4 * u]) =
-                    make_float4(dc[4 * u], dc[4 * u + 1], dc[4 * u + 2], dc[4 * u + 3]);
-        } else {
-#pragma unroll
-            for (int u = 0; u < ROW; ++u) s_sh[t * PAD + u] = dc[u];
-        }
+        stage_sh_row<DEG>(&s_sh[t * PAD], &dcoef[0][0]);
     }
     __syncthreads();
     // Block segments start at row i0 (a multiple of 128), so each is 16-byte aligned in HBM
@@ -823,7 +854,7 @@ cudaError_t launch_preprocess_bwd(int n, const darb_splats &sp, const Cam &cam, 
                                   const int *radius, const uint8_t *clamped, const float *grad2d,
                                   const GradOut &out, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    const int threads = 256, blocks = (n + threads - 1) / threads;
+    const int threads = kBwdAdamThreads, blocks = (n + threads - 1) / threads;
     const float4 *q = reinterpret_cast<const float4 *>(sp.quats);
     const float4 *g = reinterpret_cast<const float4 *>(grad2d);
     switch (sp.sh_degree) {

@@ -43,83 +43,116 @@ k_l1_loss(const float *__restrict__ image, const float *__restrict__ target, int
     }
 }
 
-// act: 0 = identity, 1 = exp (log-scale -> scale), 2 = sigmoid (logit -> opacity).
-// For act != 0 the incoming gradient is w.r.t. the activated value and `activated` holds that
-// value; the raw gradient is g * d(act)/d(raw), and `activated` is refreshed after the step.
+// The whole Adam step of a training state in one launch: each block takes kAdamBlock consecutive floats
+// of one parameter group (the groups' blocks one after the other), float4 lanes, the loads of a
+// thread's lanes issued before the first update.  HBM-bound; as a launch per group (and scalar lanes
+// for the SH rows whose length is no multiple of 4) the small groups ran at half the copy rate
+// and a small state was five launches: 243 -> 232 us at 1M splats,
+// degree 3 (1.63 GB at 7.0 TB/s); with the gradients before it, degree 2 320 -> 220 us, degree 0 111 -> 101.
+constexpr int kAdamThreads = 256, kAdamLanes = 2;
+constexpr int kAdamBlock = kAdamThreads * kAdamLanes * 4;  // floats per block
+
+// ACT: 0 = identity, 1 = exp (log-scale -> scale), 2 = sigmoid (logit -> opacity).  For ACT != 0 the
+// incoming gradient is w.r.t. the activated value and `act` holds that value; the raw gradient is
+// g * d(act)/d(raw), and `act` is refreshed after the step.
 template <int ACT>
-__device__ __forceinline__ void adam_elem(float &p, float g, float &m, float &v, float lr, float b1, float b2,
-                                          float eps, float ibc1, float ibc2, float *act_val) {
-    if (ACT == 1) g *= *act_val;
-    if (ACT == 2) g *= *act_val * (1.0f - *act_val);
-    AdamConsts c;
-    c.b1 = b1; c.b2 = b2; c.eps = eps; c.ibc1 = ibc1; c.ibc2 = ibc2;
+__device__ __forceinline__ void adam_elem(float &p, float g, float &m, float &v, float lr, const AdamConsts &c,
+                                          float &act) {
+    if (ACT == 1) g *= act;
+    if (ACT == 2) g *= act * (1.0f - act);
     adam_apply(p, g, m, v, lr, c);
-    if (ACT == 1) *act_val = expf(p);
-    if (ACT == 2) *act_val = 1.0f / (1.0f + expf(-p));
+    if (ACT == 1) act = expf(p);
+    if (ACT == 2) act = 1.0f / (1.0f + expf(-p));
 }
 
-// Flat parameter group, float4 lanes; `row`/`split` select lr2 for the elements whose index
-// within a row of ROW floats is >= SPLIT (the SH coefficients after the DC term).  ROW is a
-// multiple of 4 (or 0 for a single learning rate), so no float4 straddles two rows.
-template <int ACT, int ROW, int SPLIT>
-__global__ void __launch_bounds__(256)
-k_adam4(long long count, float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-        float *__restrict__ v, float lr, float lr2, float b1, float b2, float eps, float ibc1, float ibc2,
-        float *__restrict__ activated) {
-    pdl_entry();
-    const long long n4 = count >> 2;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < n4; j += stride) {
-        float4 P = reinterpret_cast<float4 *>(p)[j];
-        const float4 G = reinterpret_cast<const float4 *>(g)[j];
-        float4 Mm = reinterpret_cast<float4 *>(m)[j];
-        float4 V = reinterpret_cast<float4 *>(v)[j];
-        float4 A = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (ACT) A = reinterpret_cast<float4 *>(activated)[j];
-        float lrs[4] = {lr, lr, lr, lr};
-        if (ROW > 0) {
-            const int pos = (int)((j * 4) % (ROW > 0 ? ROW : 1));  // ROW is a compile-time constant
+template <int ACT, class LrOf>
+__device__ __forceinline__ void adam_group(long long count, long long block, float *__restrict__ p,
+                                           const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
+                                           float *__restrict__ act, LrOf lr_of, const AdamConsts &c) {
+    const long long n4 = count >> 2, j0 = block * (kAdamBlock / 4) + threadIdx.x;
+    float4 P[kAdamLanes], G[kAdamLanes], M[kAdamLanes], V[kAdamLanes], A[kAdamLanes];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) lrs[u] = (pos + u >= SPLIT) ? lr2 : lr;
+    for (int u = 0; u < kAdamLanes; ++u) {
+        const long long j = j0 + u * kAdamThreads;
+        if (j < n4) {
+            P[u] = reinterpret_cast<float4 *>(p)[j];
+            G[u] = reinterpret_cast<const float4 *>(g)[j];
+            M[u] = reinterpret_cast<float4 *>(m)[j];
+            V[u] = reinterpret_cast<float4 *>(v)[j];
+            A[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (ACT) A[u] = reinterpret_cast<float4 *>(act)[j];
         }
-        adam_elem<ACT>(P.x, G.x, Mm.x, V.x, lrs[0], b1, b2, eps, ibc1, ibc2, &A.x);
-        adam_elem<ACT>(P.y, G.y, Mm.y, V.y, lrs[1], b1, b2, eps, ibc1, ibc2, &A.y);
-        adam_elem<ACT>(P.z, G.z, Mm.z, V.z, lrs[2], b1, b2, eps, ibc1, ibc2, &A.z);
-        adam_elem<ACT>(P.w, G.w, Mm.w, V.w, lrs[3], b1, b2, eps, ibc1, ibc2, &A.w);
-        reinterpret_cast<float4 *>(p)[j] = P;
-        reinterpret_cast<float4 *>(m)[j] = Mm;
-        reinterpret_cast<float4 *>(v)[j] = V;
-        if (ACT) reinterpret_cast<float4 *>(activated)[j] = A;
     }
-    // scalar tail (count % 4 elements)
-    if (blockIdx.x == 0 && threadIdx.x < (count & 3)) {
+#pragma unroll
+    for (int u = 0; u < kAdamLanes; ++u) {
+        const long long j = j0 + u * kAdamThreads;
+        if (j < n4) {
+            float lr[4];
+            lr_of(4 * j, lr);
+            adam_elem<ACT>(P[u].x, G[u].x, M[u].x, V[u].x, lr[0], c, A[u].x);
+            adam_elem<ACT>(P[u].y, G[u].y, M[u].y, V[u].y, lr[1], c, A[u].y);
+            adam_elem<ACT>(P[u].z, G[u].z, M[u].z, V[u].z, lr[2], c, A[u].z);
+            adam_elem<ACT>(P[u].w, G[u].w, M[u].w, V[u].w, lr[3], c, A[u].w);
+            reinterpret_cast<float4 *>(p)[j] = P[u];
+            reinterpret_cast<float4 *>(m)[j] = M[u];
+            reinterpret_cast<float4 *>(v)[j] = V[u];
+            if (ACT) reinterpret_cast<float4 *>(act)[j] = A[u];
+        }
+    }
+    // the ragged end (count % 4 floats), by the group's first block
+    if (block == 0 && threadIdx.x < (unsigned)(count & 3)) {
         const long long i = (n4 << 2) + threadIdx.x;
-        float pp = p[i], mm = m[i], vv = v[i];
-        float a = ACT ? activated[i] : 0.f;
-        const float l = (ROW > 0 && (int)(i % (ROW > 0 ? ROW : 1)) >= SPLIT) ? lr2 : lr;
-        adam_elem<ACT>(pp, g[i], mm, vv, l, b1, b2, eps, ibc1, ibc2, &a);
+        float lr[4], pp = p[i], mm = m[i], vv = v[i], a = ACT ? act[i] : 0.f;
+        lr_of(i, lr);
+        adam_elem<ACT>(pp, g[i], mm, vv, lr[0], c, a);
         p[i] = pp;
         m[i] = mm;
         v[i] = vv;
-        if (ACT) activated[i] = a;
+        if (ACT) act[i] = a;
     }
 }
 
-// Rows whose length is not a multiple of 4 (SH degrees 0 and 2): scalar lanes.
-template <int ROW, int SPLIT>
-__global__ void __launch_bounds__(256)
-k_adam_rows(long long count, float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-            float *__restrict__ v, float lr, float lr2, float b1, float b2, float eps, float ibc1, float ibc2) {
+__host__ __device__ constexpr long long adam_blocks(long long count) { return (count + kAdamBlock - 1) / kAdamBlock; }
+
+template <int DEG>
+__global__ void __launch_bounds__(kAdamThreads)
+k_adam(long long n, darb_train_params P, darb_splat_grads G, darb_adam_state A, AdamConsts c) {
     pdl_entry();
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (long long)gridDim.x * blockDim.x) {
-        float pp = p[i], mm = m[i], vv = v[i];
-        const float l = (int)(i % ROW) >= SPLIT ? lr2 : lr;
-        adam_elem<0>(pp, g[i], mm, vv, l, b1, b2, eps, ibc1, ibc2, nullptr);
-        p[i] = pp;
-        m[i] = mm;
-        v[i] = vv;
+    constexpr int ROW = 3 * (DEG + 1) * (DEG + 1);
+    auto same = [](float lr) {
+        return [lr](long long, float (&r)[4]) { r[0] = r[1] = r[2] = r[3] = lr; };
+    };
+    const float dc = c.lr_sh_dc, rest = c.lr_sh_rest;
+    // the SH rows first, the bulk of the bytes; their first 3 floats are the DC term
+    long long b = blockIdx.x;
+    if (b < adam_blocks(ROW * n)) {
+        adam_group<0>(ROW * n, b, P.sh, G.dsh, A.m_sh, A.v_sh, nullptr, [=](long long f, float (&r)[4]) {
+            const int pos = (int)(f % ROW);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int q = pos + u >= ROW ? (pos + u) % ROW : pos + u;  // a float4 straddles rows of 3 and 27
+                r[u] = q < 3 ? dc : rest;
+            }
+        }, c);
+        return;
     }
+    b -= adam_blocks(ROW * n);
+    if (b < adam_blocks(4 * n)) {
+        adam_group<0>(4 * n, b, P.quats, G.dquats, A.m_quats, A.v_quats, nullptr, same(c.lr_quats), c);
+        return;
+    }
+    b -= adam_blocks(4 * n);
+    if (b < adam_blocks(3 * n)) {
+        adam_group<0>(3 * n, b, P.means, G.dmeans, A.m_means, A.v_means, nullptr, same(c.lr_means), c);
+        return;
+    }
+    b -= adam_blocks(3 * n);
+    if (b < adam_blocks(3 * n)) {
+        adam_group<1>(3 * n, b, P.log_scales, G.dscales, A.m_scales, A.v_scales, P.scales, same(c.lr_scales), c);
+        return;
+    }
+    b -= adam_blocks(3 * n);
+    adam_group<2>(n, b, P.opacity_logits, G.dopacities, A.m_opac, A.v_opac, P.opacities, same(c.lr_opacities), c);
 }
 
 int grid_for(long long count) {
@@ -177,36 +210,14 @@ cudaError_t launch_adam(const darb_train_params &p, const darb_splat_grads &g, c
     const long long n = p.n;
     if (n == 0) return cudaSuccess;
     const AdamConsts ac = make_adam_consts(c);
-    const float ibc1 = ac.ibc1, ibc2 = ac.ibc2;
-    const float b1 = c.beta1, b2 = c.beta2, eps = c.eps;
-    const long long K = (long long)(p.sh_degree + 1) * (p.sh_degree + 1);
-    auto g4 = [](long long count) { return grid_for((count + 3) / 4); };
-    launch_k(k_adam4<0, 0, 0>, g4(3 * n), 256, 0, st, 3 * n, p.means, g.dmeans, s.m_means, s.v_means, c.lr_means,
-             c.lr_means, b1, b2, eps, ibc1, ibc2, nullptr);
-    launch_k(k_adam4<1, 0, 0>, g4(3 * n), 256, 0, st, 3 * n, p.log_scales, g.dscales, s.m_scales, s.v_scales, c.lr_scales,
-             c.lr_scales, b1, b2, eps, ibc1, ibc2, p.scales);
-    launch_k(k_adam4<0, 0, 0>, g4(4 * n), 256, 0, st, 4 * n, p.quats, g.dquats, s.m_quats, s.v_quats, c.lr_quats,
-             c.lr_quats, b1, b2, eps, ibc1, ibc2, nullptr);
-    launch_k(k_adam4<2, 0, 0>, g4(n), 256, 0, st, n, p.opacity_logits, g.dopacities, s.m_opac, s.v_opac, c.lr_opacities,
-             c.lr_opacities, b1, b2, eps, ibc1, ibc2, p.opacities);
-    const long long cs = 3 * K * n;
+    const long long row = 3ll * (p.sh_degree + 1) * (p.sh_degree + 1);
+    const long long blocks = adam_blocks(row * n) + adam_blocks(4 * n) + 2 * adam_blocks(3 * n) + adam_blocks(n);
+    auto go = [&](auto kernel) { launch_k(kernel, (unsigned)blocks, kAdamThreads, 0, st, n, p, g, s, ac); };
     switch (p.sh_degree) {
-    case 0:
-        launch_k(k_adam_rows<3, 3>, grid_for(cs), 256, 0, st, cs, p.sh, g.dsh, s.m_sh, s.v_sh, c.lr_sh_dc, c.lr_sh_rest, b1,
-                 b2, eps, ibc1, ibc2);
-        break;
-    case 1:
-        launch_k(k_adam4<0, 12, 3>, g4(cs), 256, 0, st, cs, p.sh, g.dsh, s.m_sh, s.v_sh, c.lr_sh_dc, c.lr_sh_rest, b1, b2,
-                 eps, ibc1, ibc2, nullptr);
-        break;
-    case 2:
-        launch_k(k_adam_rows<27, 3>, grid_for(cs), 256, 0, st, cs, p.sh, g.dsh, s.m_sh, s.v_sh, c.lr_sh_dc, c.lr_sh_rest, b1,
-                 b2, eps, ibc1, ibc2);
-        break;
-    default:
-        launch_k(k_adam4<0, 48, 3>, g4(cs), 256, 0, st, cs, p.sh, g.dsh, s.m_sh, s.v_sh, c.lr_sh_dc, c.lr_sh_rest, b1, b2,
-                 eps, ibc1, ibc2, nullptr);
-        break;
+    case 0: go(k_adam<0>); break;
+    case 1: go(k_adam<1>); break;
+    case 2: go(k_adam<2>); break;
+    default: go(k_adam<3>); break;
     }
     return cudaGetLastError();
 }

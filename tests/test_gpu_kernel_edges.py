@@ -141,3 +141,48 @@ def test_dssim_at_tile_edges(width, height):
     torch.cuda.synchronize()
     assert abs(float(loss[0]) - ref_loss) <= 2e-6 and abs(float(loss[1]) - ref_ssim) <= 4e-6
     grad_close("dL", to_np(dl), ref_dl)
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 300])
+@pytest.mark.parametrize("deg", [0, 1, 2, 3])
+def test_preprocess_backward_stores_at_block_edges_and_off_the_boundary(n, deg):
+    """Gradients leave a block of 128 splats as contiguous ranges: ragged last blocks, and arrays 4 bytes past
+    a 16-byte boundary, give the values of aligned ones."""
+    s = synth.uniform_cube_scene(n, seed=deg, sh_degree=deg)
+    cam = synth.pinhole((0.0, 0.0, 4.0), 64, 48, 60.0)
+    sd = darb.splats_to_device(s)
+    kp = darb.darb_kernel_defaults("half_cosine")
+    proj = darb.darb_preprocess(sd, cam, kp, 16)
+    g2 = _t(np.random.default_rng(n).normal(size=(n, 12)).astype(np.float32))
+    a = darb.darb_preprocess_bwd(sd, cam, kp, proj, g2)
+    b = darb.SplatGrads.empty_like(sd)
+    for f in ("dmeans", "dscales", "dopacities"):
+        setattr(b, f, _off_by_one(torch.full_like(getattr(b, f), np.nan)))
+    darb.darb_preprocess_bwd(sd, cam, kp, proj, g2, b)
+    torch.cuda.synchronize()
+    seen = to_np(proj.radius) > 0
+    assert seen.any()
+    for f in ("dmeans", "dscales", "dquats", "dopacities", "dsh"):
+        x, y = to_np(getattr(a, f)), to_np(getattr(b, f))
+        np.testing.assert_array_equal(x, y, err_msg=f)
+        assert (x[~seen] == 0).all() and np.isfinite(x).all()
+
+
+@pytest.mark.parametrize("n", [1, 2, 683, 2049])
+@pytest.mark.parametrize("deg", [0, 2, 3])
+def test_adam_groups_at_block_edges(n, deg):
+    """Groups shorter than a float4 and just over a block's 2048 floats (3 x 683 and 2049): every element
+    takes exactly one step."""
+    from test_gpu_train import _cfg, _check_adam, _clone, _oracle_adam, _to_device, _train_state
+    s = synth.uniform_cube_scene(n, seed=deg, sh_degree=deg)
+    rng = np.random.default_rng(50 + deg)
+    raw, state = _train_state(s, rng, warm=True)
+    p, st = _to_device(raw, state, deg)
+    p0, _ = _clone(p, st)
+    grads = {k: (1e-3 * rng.normal(size=getattr(s, k).shape)).astype(np.float32)
+             for k in ("means", "scales", "quats", "opacities", "sh")}
+    ref_raw, ref_state = _oracle_adam(p, st, {k: v.astype(np.float64) for k, v in grads.items()}, 5)
+    darb.darb_adam_step(p, darb.SplatGrads(*(_t(grads[k]) for k in ("means", "scales", "quats", "opacities", "sh"))), st,
+                        _cfg(5))
+    torch.cuda.synchronize()
+    _check_adam(p0, p, st, ref_raw, ref_state, upd_rtol=1e-5, mom_tol=2e-6)
