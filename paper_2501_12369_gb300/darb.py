@@ -166,6 +166,8 @@ def library_path() -> str:
 def lib() -> ctypes.CDLL:
     """Load libdarb.so (built in-tree by paper_2501_12369_gb300.build).  Raises if it is missing."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = library_path()
@@ -192,12 +194,13 @@ def _check(status: int, where: str):
 
 
 def _p(t):
-    return None if t is None else c_vp(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return c_vp(s.cuda_stream)
+    if stream is None:  # the current stream's handle, without a torch.cuda.Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 # ---------------------------------------------------------------------------
@@ -245,7 +248,8 @@ def darb_kernel_psi(kp: darb_kernel_params, device="cuda", stream=None) -> float
 def camera(cam) -> darb_camera:
     """darb_camera from any object with viewmat, fx, fy, cx, cy, near, width, height, bg."""
     c = darb_camera()
-    c.viewmat[:] = [float(v) for v in np.asarray(cam.viewmat, np.float32).reshape(16)]
+    view = np.ascontiguousarray(cam.viewmat, np.float32).reshape(16)
+    ctypes.memmove(c.viewmat, view.ctypes.data, 64)
     c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
     c.near_plane = float(cam.near)
     c.width, c.height = int(cam.width), int(cam.height)
@@ -308,7 +312,8 @@ class Projected:
                          torch.empty(n, dtype=torch.int64, **f))
 
     def struct(self) -> darb_projected:
-        return darb_projected(*(_p(getattr(self, f.name)) for f in dataclasses.fields(self)))
+        return darb_projected(_p(self.depth), _p(self.radius), _p(self.tile_rect), _p(self.mean2d), _p(self.conic_o),
+                              _p(self.rgb), _p(self.clamped), _p(self.tiles_touched), _p(self.tile_runs))
 
 
 @dataclasses.dataclass
@@ -381,8 +386,9 @@ def darb_bin_sort(proj: Projected, n, tile, cam, workspace: torch.Tensor, capaci
                   sync=True, stream=None, strategy=DARB_SORT_DEPTH_THEN_TILE, kparams=None):
     """sync=True reads M back (one stream synchronisation) and sizes the sort by it.  kparams:
     the kernel the records were projected with (default: the one darb_preprocess recorded)."""
-    tx, ty = darb_tile_grid(cam, tile)
-    out = Binning.empty(capacity, tx * ty, workspace.device) if out is None else out
+    if out is None:
+        tx, ty = darb_tile_grid(cam, tile)
+        out = Binning.empty(capacity, tx * ty, workspace.device)
     pr, c, b = proj.struct(), camera(cam), out.struct()
     kp = proj.kparams if kparams is None else kparams
     m = ctypes.c_uint64(0)
@@ -400,8 +406,9 @@ def darb_bin_sort(proj: Projected, n, tile, cam, workspace: torch.Tensor, capaci
 def darb_bin_sort_noalloc(proj: Projected, n, tile, cam, capacity, out: Binning | None = None, sync=True,
                           stream=None, kparams=None):
     """darb_bin_sort with the library's static device scratch instead of a caller workspace."""
-    tx, ty = darb_tile_grid(cam, tile)
-    out = Binning.empty(capacity, tx * ty, proj.depth.device) if out is None else out
+    if out is None:
+        tx, ty = darb_tile_grid(cam, tile)
+        out = Binning.empty(capacity, tx * ty, proj.depth.device)
     pr, c, b = proj.struct(), camera(cam), out.struct()
     kp = proj.kparams if kparams is None else kparams
     m = ctypes.c_uint64(0)
@@ -578,6 +585,7 @@ class Rasterizer:
             self.kparams.psi = float(psi)
         self.device = device
         self.tiles_x, self.tiles_y = darb_tile_grid(cam, tile)
+        self._size = (cam.width, cam.height)
         self.capacity = int(capacity) if capacity else 0
         self._ws = None
         self._bins = None
@@ -592,13 +600,20 @@ class Rasterizer:
             self._n = n
 
     def _sort(self, proj, n, owned):
-        tx, ty = darb_tile_grid(self.cam, self.tile)
-        if (tx, ty) != (self.tiles_x, self.tiles_y):  # the camera was changed to another resolution
-            self.tiles_x, self.tiles_y = tx, ty
-            self._ws = None
+        if (self.cam.width, self.cam.height) != self._size:
+            tx, ty = darb_tile_grid(self.cam, self.tile)
+            self._size = (self.cam.width, self.cam.height)
+            if (tx, ty) != (self.tiles_x, self.tiles_y):  # the camera was changed to another resolution
+                self.tiles_x, self.tiles_y = tx, ty
+                self._ws = None
         self._ensure(n, self.capacity)
-        out = (Binning.empty(self.capacity, tx * ty, self.device, keys=self.strategy == DARB_SORT_KEYS64)
-               if owned else self._bins)
+        out = self._bins
+        if owned:  # the sort writes the count and the status itself: no fill launches
+            f = dict(device=self.device)
+            keys = torch.empty(self.capacity, dtype=torch.int64, **f) if self.strategy == DARB_SORT_KEYS64 else None
+            words = torch.empty(8, dtype=torch.int32, **f)  # each on its own 16 bytes
+            out = Binning(keys, torch.empty(self.capacity, dtype=torch.int32, **f),
+                          torch.empty(self.tiles_x * self.tiles_y, 2, dtype=torch.int32, **f), words[:1], words[4:5])
         return darb_bin_sort(proj, n, self.tile, self.cam, self._ws, self.capacity, out, sync=self.sync,
                              strategy=self.strategy)
 
