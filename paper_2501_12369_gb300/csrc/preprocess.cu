@@ -237,7 +237,7 @@ __device__ __forceinline__ bool project_fixed(const float m[3], const float s[3]
 // its projected geometry, in shared memory.  Phase 2: the threads take the queued (visible)
 // splats densely and do the heavy part -- member tiles by row runs, SH colour, the records --
 // so that whole warps, not 38% of each warp's lanes, run it.
-constexpr int kPreThreads = 256;
+constexpr int kPreThreads = 128;
 
 // L2 prefetch of a queued splat's SH row in phase 1 (1), or none (0).
 #ifndef DARB_PRE_SH_PREFETCH
@@ -265,14 +265,14 @@ struct PreGeom {
     int radius, idx;
 };
 
-// Compiled for 5 resident CTAs per SM (48 registers, 1280 threads, each with DARB_PRE_SPT = 2
-// splats): the projection is latency-bound, and a register cap raised occupancy from the
-// compiler's choice (0.172 -> 0.153 ms at 3M splats / 1080p with 8 CTAs of one splat per thread).
-// With two splats per thread, 5 CTAs measure 0.136 ms against 0.145 at 6 (40 registers, which
-// spill) and 0.142 at 4; one splat per thread at 6 CTAs: 0.145.  DARB_PRE_MIN_CTAS=0 leaves the
-// register count to the compiler.
+// Compiled for 9 resident CTAs per SM (48 registers, 1152 threads, each with DARB_PRE_SPT = 2
+// splats): the projection is latency-bound.  Small CTAs end sooner once their queue, some 40% of the
+// splats, no longer fills every warp: 1M splats, 1080p, 32-pixel tiles (16-pixel; 3M splats): 54.6
+// (71.6; 136) us with 5 CTAs of 256 threads, 52.5 (68.8; 130) with 10 of 128, 51.7 (68.7; 129) with 9,
+// 56.8 (73.1; 139) with 12, 52.9 (71.5; 133) with 20 of 64; three and four splats a thread 57 and 78.
+// DARB_PRE_MIN_CTAS=0 leaves the register count to the compiler.
 #ifndef DARB_PRE_MIN_CTAS
-#define DARB_PRE_MIN_CTAS 5
+#define DARB_PRE_MIN_CTAS 9
 #endif
 // Splats per thread of k_preprocess: with 2, a thread issues both splats' loads before it
 // projects the first.
