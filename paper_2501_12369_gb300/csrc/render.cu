@@ -126,17 +126,78 @@ struct FwdSink {
 
 // The L1 image loss (Sec. 4.2) taken in the forward's epilogue, where each pixel's colour is
 // in registers: dL/dC = sign(C - target) / count per channel, and the block's sum of
-// |C - target| / count added to *loss (zeroed by the caller).
+// |C - target| / count added to *loss (zeroed by the caller).  FP32 additions in memory round at
+// the size of the whole sum, so there should be few: the CTAs of a cluster of kL1Cluster hand their sums
+// to its first one, which adds them at once (1 020 additions for 1080p in 32-pixel tiles instead of
+// 8 160, whose error reached 2e-6 of the loss).  Only the first CTA waits for the others.
 struct L1Out {
     const float *target;
     float *dL;
     float *loss;
     float inv_count;
 };
+constexpr unsigned kL1Cluster = 8;
+
+struct L1Smem {
+    uint64_t full;  // mbarrier of the cluster's first CTA: one arrival from each of the others
+    float part[kL1Cluster];
+};
+
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// Before the compositing: the barrier is there and the cluster's CTAs run once l1_cluster_add waits.
+__device__ __forceinline__ void l1_cluster_begin(L1Smem &sm) {
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&sm.full)), "r"(kL1Cluster - 1) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+
+// Adds the cluster's sums to *loss; `sum` is thread 0's.
+__device__ __forceinline__ void l1_cluster_add(L1Smem &sm, float sum, const L1Out &l1) {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (threadIdx.x != 0) return;
+    const unsigned rank = blockIdx.x % kL1Cluster;
+    if (rank != 0) {
+        asm volatile(
+            "{\n\t"
+            ".reg .b32 part, full;\n\t"
+            "mapa.shared::cluster.u32 part, %0, 0;\n\t"
+            "mapa.shared::cluster.u32 full, %1, 0;\n\t"
+            "st.shared::cluster.f32 [part], %2;\n\t"
+            "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [full];\n\t"
+            "}" ::"r"(smem_addr(&sm.part[rank])), "r"(smem_addr(&sm.full)), "f"(sum)
+            : "memory");
+        return;
+    }
+    unsigned long long t0, now;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    for (;;) {
+        unsigned done;
+        asm volatile(
+            "{\n\t"
+            ".reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t"
+            "}" : "=r"(done) : "r"(smem_addr(&sm.full)) : "memory");
+        if (done) break;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+        if (now - t0 > 60000000000ull) {  // a minute: the other CTAs never came; the loss says so
+            atomicAdd(l1.loss, __int_as_float(0x7fc00000));
+            return;
+        }
+    }
+#pragma unroll
+    for (unsigned c = 1; c < kL1Cluster; ++c) sum += sm.part[c];
+    atomicAdd(l1.loss, sum * l1.inv_count);
+}
 
 // One tile of one view, by the whole CTA.  sink() is called once, after the compositing loop,
 // so the output pointers need not stay live in registers across it.  With L1 the epilogue also
-// takes the L1 loss of the tile's pixels (every thread of the CTA reaches it).  AUX: the outputs
+// takes the sum of the L1 loss over the square's pixels (thread 0's *l1_sum).  AUX: the outputs
 // beside the image and T that the caller may ask for (0: none, 1: last, 2: last and n_contrib).
 //
 // The body is branch-free and keeps few instructions on the ALU pipe (compares, selects, minimum),
@@ -158,7 +219,7 @@ __device__ __forceinline__ void render_tile_fwd(int item, FwdSmem<S::NT> &sm,
                                                 const float4 *__restrict__ conic_o, const float *__restrict__ rgb,
                                                 int W, int H, int tiles_x, float qmax, int strict,
                                                 const KernelSpec &ks, SinkFn sink, const L1Out &l1 = L1Out{},
-                                                float *s_l1 = nullptr) {
+                                                float *s_l1 = nullptr, float *l1_sum = nullptr) {
     constexpr int TILE = S::TILE, NT = S::NT, PIX = S::PIX, L = PIX % 2 == 0 ? 2 : 1, NV = PIX / L;  // NV groups of L lanes
     using V = Lanes<L>;
     using VT = typename V::T;
@@ -283,7 +344,7 @@ __device__ __forceinline__ void render_tile_fwd(int item, FwdSmem<S::NT> &sm,
         if (threadIdx.x == 0) {
             float sum = 0.0f;
             for (int w = 0; w < S::NT / 32; ++w) sum += s_l1[w];
-            atomicAdd(l1.loss, sum * l1.inv_count);
+            *l1_sum = sum;
         }
     }
 }
@@ -294,14 +355,26 @@ k_render_fwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ valu
              const float2 *__restrict__ mean2d, const float4 *__restrict__ conic_o,
              const float *__restrict__ rgb, int W, int H, int tiles_x, float qmax, int strict, KernelSpec ks, Bg bg,
              float *__restrict__ image, float *__restrict__ t_final, uint32_t *__restrict__ last,
-             uint32_t *__restrict__ n_contrib, L1Out l1) {
-    pdl_entry();
+             uint32_t *__restrict__ n_contrib, int n_items, L1Out l1) {
     using S = typename FwdOf<TILE>::S;
     __shared__ FwdSmem<S::NT> sm;
     __shared__ float s_l1[L1 ? (S::NT + 31) / 32 : 1];
-    render_tile_fwd<KIND, S, AUX, L1 ? kStepL1 : kStepPlain, L1>(
-        blockIdx.x, sm, ranges, values, mean2d, conic_o, rgb, W, H, tiles_x, qmax, strict, ks,
-        [&] { return FwdSink{image, t_final, last, n_contrib, bg}; }, l1, s_l1);
+    auto tile = [&](float *l1_sum) {
+        render_tile_fwd<KIND, S, AUX, L1 ? kStepL1 : kStepPlain, L1>(
+            blockIdx.x, sm, ranges, values, mean2d, conic_o, rgb, W, H, tiles_x, qmax, strict, ks,
+            [&] { return FwdSink{image, t_final, last, n_contrib, bg}; }, l1, s_l1, l1_sum);
+    };
+    if constexpr (L1) {
+        __shared__ L1Smem s_cluster;
+        l1_cluster_begin(s_cluster);
+        pdl_entry();
+        float sum = 0.0f;
+        if ((int)blockIdx.x < n_items) tile(&sum);  // the grid is whole clusters
+        l1_cluster_add(s_cluster, sum, l1);
+    } else {
+        pdl_entry();
+        tile(nullptr);
+    }
 }
 
 // Several views in one persistent launch: CTAs take items (a square of a tile of a view) from a
@@ -632,9 +705,12 @@ cudaError_t fwd_t(int n_tiles, const uint2 *ranges, const uint32_t *values, cons
                   const KernelSpec &ks, float *image, float *t_final, uint32_t *last, uint32_t *n_contrib,
                   const L1Out &l1, cudaStream_t st) {
     using S = typename FwdOf<TILE>::S;
+    const int items = n_tiles * S::PARTS;
+    const unsigned cluster = l1.target ? kL1Cluster : 1;
     auto go = [&](auto kernel) {
-        launch_k(kernel, n_tiles * S::PARTS, S::NT, 0, st, ranges, values, mean2d, conic_o, rgb, cam.W, cam.H,
-                 tiles_x, qmax, strict, ks, Bg{cam.bg[0], cam.bg[1], cam.bg[2]}, image, t_final, last, n_contrib, l1);
+        launch_cluster(kernel, (items + cluster - 1) / cluster * cluster, cluster, S::NT, 0, st, ranges, values, mean2d,
+                       conic_o, rgb, cam.W, cam.H, tiles_x, qmax, strict, ks, Bg{cam.bg[0], cam.bg[1], cam.bg[2]},
+                       image, t_final, last, n_contrib, items, l1);
     };
     if (!l1.target) go(k_render_fwd<KIND, TILE, 2, false>);
     else if (n_contrib) go(k_render_fwd<KIND, TILE, 2, true>);

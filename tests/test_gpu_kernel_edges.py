@@ -186,3 +186,21 @@ def test_adam_groups_at_block_edges(n, deg):
                         _cfg(5))
     torch.cuda.synchronize()
     _check_adam(p0, p, st, ref_raw, ref_state, upd_rtol=1e-5, mom_tol=2e-6)
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("width,height", [(1, 1), (128, 16), (16, 129), (333, 207)])
+def test_l1_epilogue_loss_at_cluster_edges(width, height, tile):
+    """Fewer CTAs than a cluster of 8, whole clusters and a last one that is not full.  Every thread adds at most
+    12 terms, and no term goes through more than 12 + 5 + 8 + 8 additions before those in memory (at
+    most 135 clusters): (33 + 135) 2^-24 < 1.1e-5 of the loss, whose terms are all positive."""
+    s = synth.uniform_cube_scene(300, seed=6)
+    cam = synth.pinhole((0.5, 0.4, 6.0), width, height, 0.8 * max(width, 24), bg=(0.2, 0.1, 0.4))
+    r, sd, proj, bins, img = gpu_forward(s, cam, "gaussian", tile)
+    target = _t(synth.random_target(height, width, seed=9))
+    out, dl, loss = darb.darb_render_fwd_l1(proj, bins, cam, r.kparams, tile, target)
+    torch.cuda.synchronize()
+    d = to_np(out.image).astype(np.float64) - to_np(target)
+    assert abs(float(loss[0]) - np.abs(d).mean()) <= 1.1e-5 * np.abs(d).mean()
+    np.testing.assert_array_equal(to_np(out.image), to_np(img.image))
+    np.testing.assert_array_equal(to_np(dl), np.sign(d).astype(np.float32) * np.float32(1.0 / (3.0 * width * height)))
