@@ -507,46 +507,63 @@ __device__ __forceinline__ bool may_reach(float A, float B, float C, float xl, f
 // T_k (g . c_k) - (g . S) / (1 - alpha_k), and g . S grows by (g . c_k) alpha_k T_k per splat,
 // so each pixel carries the scalar g . S instead of three colour channels.
 //
-// One warp per CTA takes a block of LX x (32 / LX * PIX) pixels, PIX of one column a lane, and walks
-// the tile's run 32 records at a time: each lane gathers one, keeps it if its ellipse may reach
-// the block, and the kept ones are compacted in shared memory.  No barrier beyond the warp and
-// no shared-memory atomics.  The pair body is branch-free (a pair that does not contribute has
-// alpha 0 and leaves T, g . S and every sum as they are) and runs on pairs of pixels with the
-// packed two-lane FP32 instructions.  The gradients w.r.t. centre and conic are sums of s, s dy and
-// s dy^2 over a lane's column (s = dL/dF dF/dq) times powers of the shared dx: three sums a pair
-// instead of five products, with the conic's factors applied once per record.  The warp's nine
-// sums per record leave through vector atomics, a lane per record.
+// A CTA of NW warps takes a tile, a warp of it a block of LX x (32 / LX * PIX) pixels, PIX of one
+// column a lane.  The warps walk the tile's run independently, 32 records at a
+// time: each lane gathers one, keeps it if its ellipse may reach the block, and the kept ones are
+// compacted in the warp's shared memory.  The pair body is branch-free (a pair that does not
+// contribute has alpha 0 and leaves T, g . S and every sum as they are) and runs on pairs of pixels
+// with the packed two-lane FP32 instructions.  The gradients w.r.t. centre and conic are sums of s,
+// s dy and s dy^2 over a lane's column (s = dL/dF dF/dq) times powers of the shared dx: three sums a
+// pair instead of five products, with the conic's factors applied once per record.
 //
-// Bound by the FP32 and ALU pipes together (two thirds of the issue slots, 50 slots per 32 pairs
-// with the sinc's two series, 88-100 before).  Mod. sinc, 300k splats, 1245 x 825, 16-pixel tiles:
-// 217 us with a CTA per tile, branches per pair and nine products, 127 with eight pixels a lane,
-// 113 with four, 126 with two; half-cosine 100 / 59 / 58 / 75; Gaussian 367 / 228 / 199 / 214; on
-// 32-pixel tiles 273 / 130 / 117 / 130; 8-pixel tiles (8 x 8 blocks, two pixels) 237 -> 118.
-template <int KIND, int LX, int PIX>
-__global__ void __launch_bounds__(32, 24)
+// The sums are kept per warp in shared memory for a window of kWindow records, added over the CTA at
+// the window's end, and leave through one set of vector atomics per (tile, record): a near splat
+// that covers the image then sums as few FP32 terms in memory as there are tiles.  A set per
+// block instead took 114 us where this takes 122, but made the error of such sums 2.7 times as
+// large.  Windows of 64 cost 1% more; of 96 in CTAs of eight warps, within 48 KB.
+//
+// Bound by the FP32 and ALU pipes of the pair body.  Launch, 300k splats, 1245 x 825, 16-pixel tiles, against
+// a thread per pixel column of the tile with scalar arithmetic and a list of kept records for the
+// whole CTA: sinc 217 -> 122 us, Gaussian 367 -> 225, half-cosine 100 -> 64; sinc with 32-pixel tiles
+// 273 -> 135, 8-pixel 237 -> 120; 20k splats 142 -> 84, at 333 x 207 167 -> 67.
+template <int KIND, int LX, int PIX, int NW>
+__global__ void __launch_bounds__(32 * NW, (PIX == 2 ? 28 : NW == 8 ? 24 : 20) / NW)
 k_render_bwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ values,
              const float2 *__restrict__ mean2d, const float4 *__restrict__ conic_o,
              const float *__restrict__ rgb, int W, int H, int tiles_x, int tile, float qmax, int strict, KernelSpec ks,
              Bg bg, const float *__restrict__ t_final, const uint32_t *__restrict__ last,
              const float *__restrict__ dL_dimage, float4 *__restrict__ grad2d) {
     pdl_entry();
-    constexpr int LY = 32 / LX, BH = LY * PIX, NV = PIX / 2;
-    __shared__ float4 s_a[32], s_b[32];            // x, y, A, 2B; C, opacity, red, green
-    __shared__ float s_c[32];                      // blue
-    __shared__ int s_pos[32];
-    __shared__ uint32_t s_id[32];
-    __shared__ float s_sum[32][9];
-    const int lane = threadIdx.x;
-    const int px_parts = tile / LX, parts = px_parts * (tile / BH);
-    const int t = blockIdx.x / parts, part = blockIdx.x % parts;
-    const int x0 = (t % tiles_x) * tile + part % px_parts * LX, y0 = (t / tiles_x) * tile + part / px_parts * BH;
-    const int px = x0 + lane % LX;
-    const float fpx = (float)px + 0.5f;
-    const int start = (int)ranges[t].x;
+    constexpr int LY = 32 / LX, BH = LY * PIX, NV = PIX / 2, kWindow = NW == 8 ? 96 : 128;
+    struct WarpSmem {
+        float4 a[32], b[32];      // x, y, A, 2B; C, opacity, red, green
+        float c[32];              // blue
+        int pos[32];
+        float sum[kWindow * 9];
+    };
+    __shared__ WarpSmem smem[NW];
+    __shared__ int s_last[NW];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    WarpSmem &sm = smem[warp];
+    const int t = blockIdx.x, start = (int)ranges[t].x;
     const uint32_t qlim = __float_as_uint(support_limit(qmax, strict));
     const size_t plane = (size_t)W * H;
     auto dup = [](float a) { return make_float2(a, a); };
-
+    auto emit = [&](uint32_t id, float4 co, const float (&s)[9]) {  // a record's sums to its gradients
+        bool any = false;
+#pragma unroll
+        for (int u = 0; u < 9; ++u) any |= s[u] != 0.0f;
+        if (!any) return;
+        const float A = co.x, B = co.y, C = co.z, o = co.w;
+        float4 *gp = grad2d + 3 * (size_t)id;
+        atomicAdd(gp, make_float4(2.0f * o * (A * s[0] + B * s[1]), 2.0f * o * (B * s[0] + C * s[1]), o * s[2],
+                                  2.0f * o * s[3]));
+        atomicAdd(gp + 1, make_float4(o * s[4], s[5], s[6], s[7]));
+        atomicAdd(reinterpret_cast<float *>(gp + 2), s[8]);
+    };
+    const int x0 = (t % tiles_x) * tile + warp % (tile / LX) * LX, y0 = (t / tiles_x) * tile + warp / (tile / LX) * BH;
+    const int px = x0 + lane % LX;
+    const float fpx = (float)px + 0.5f;
     float2 nfpy[NV], T[NV], GS[NV], g0[NV], g1[NV], g2[NV];
     int my_last[PIX], nlast = 0;
 #pragma unroll
@@ -576,126 +593,138 @@ k_render_bwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ valu
         }
     }
     nlast = (int)__reduce_max_sync(0xffffffffu, (unsigned)nlast);
+    if (lane == 0) s_last[warp] = nlast;
     // an upstream gradient that is not finite reaches only the splats that its pixel blended
     bool odd = false;
 #pragma unroll
     for (int v = 0; v < NV; ++v)
-        odd |= !(isfinite(g0[v].x) && isfinite(g0[v].y) && isfinite(g1[v].x) && isfinite(g1[v].y) && isfinite(g2[v].x) &&
-                 isfinite(g2[v].y));
+        odd |= !(isfinite(g0[v].x) && isfinite(g0[v].y) && isfinite(g1[v].x) && isfinite(g1[v].y) &&
+                 isfinite(g2[v].x) && isfinite(g2[v].y));
     odd = __any_sync(0xffffffffu, odd);
-    for (int bend = nlast; bend > 0; bend -= 32) {
-        const int pos = bend - 1 - lane;  // lane 0 the last record: the walk goes back to front
-        bool keep = false;
-        uint32_t id = 0;
-        float2 xy;
-        float4 co;
-        if (pos >= 0) {
-            id = values[start + pos];
-            xy = mean2d[id];
-            co = conic_o[id];
-            keep = may_reach(co.x, co.y, co.z, (float)x0 + 0.5f - xy.x, (float)(x0 + LX) - 0.5f - xy.x,
-                             (float)y0 + 0.5f - xy.y, (float)(y0 + BH) - 0.5f - xy.y, qmax);
-        }
-        const uint32_t kept = __ballot_sync(0xffffffffu, keep);
-        const int n = __popc(kept);
-        if (keep) {
-            const int slot = __popc(kept & ((1u << lane) - 1u));
-            s_a[slot] = make_float4(xy.x, xy.y, co.x, 2.0f * co.y);
-            s_b[slot] = make_float4(co.z, co.w, rgb[3 * (size_t)id], rgb[3 * (size_t)id + 1]);
-            s_c[slot] = rgb[3 * (size_t)id + 2];
-            s_pos[slot] = pos;
-            s_id[slot] = id;
-        }
-        __syncwarp();
-        auto walk = [&](int j, auto masked) {
-            const float4 ra = s_a[j], rb = s_b[j];
-            const float rc = s_c[j];
-            const int rpos = s_pos[j];
-            const float dx1 = __fsub_rn(ra.x, fpx);
-            const float2 dx = dup(dx1), y = dup(ra.y), A = dup(ra.z), B2 = dup(ra.w), Cc = dup(rb.x), o = dup(rb.y);
-            const float2 c0 = dup(rb.z), c1 = dup(rb.w), c2 = dup(rc);
-            float2 S0 = dup(0.0f), S1 = dup(0.0f), S2 = dup(0.0f), SF = dup(0.0f), W0 = dup(0.0f), W1 = dup(0.0f),
-                   W2 = dup(0.0f);
+    __syncthreads();
+    int top = nlast;
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const float2 dy = __fadd2_rn(y, nfpy[v]);
-                const float2 e = __ffma2_rn(A, dx, __fmul2_rn(B2, dy));  // conic_q
-                const float2 qr = __ffma2_rn(dx, e, __fmul2_rn(__fmul2_rn(Cc, dy), dy));
-                // outside the support the profile is taken at its limit: finite, so that the pair's zero
-                // weight leaves the sums alone (as unsigned words negative values lie above the limit too)
-                const uint32_t q0 = __float_as_uint(qr.x), q1 = __float_as_uint(qr.y);
-                const float2 q = make_float2(__uint_as_float(min(q0, qlim)), __uint_as_float(min(q1, qlim)));
-                float2 F, dF;
-                if constexpr (KIND == DARB_GENERIC) {  // costly: skipped where no lane is in the support
-                    F = dF = dup(0.0f);
-                    if (__any_sync(0xffffffffu, q0 <= qlim || q1 <= qlim)) {
-                        generic_both(q.x, ks, F.x, dF.x);
-                        generic_both(q.y, ks, F.y, dF.y);
+    for (int w = 0; w < NW; ++w) top = max(top, s_last[w]);
+#pragma unroll 1
+    for (int win = top > 0 ? (top - 1) / kWindow * kWindow : -1; win >= 0; win -= kWindow) {
+        const int end = min(top - win, kWindow);
+        for (int i = lane; i < 9 * end; i += 32) sm.sum[i] = 0.0f;
+        int bstart;
+        for (int bend = min(nlast, win + kWindow); bend > win; bend = bstart) {
+            bstart = max(bend - 32, win);
+            const int pos = bend - 1 - lane;  // lane 0 the last record: the walk goes back to front
+            bool keep = false;
+            uint32_t id = 0;
+            float2 xy;
+            float4 co;
+            if (pos >= bstart) {
+                id = values[start + pos];
+                xy = mean2d[id];
+                co = conic_o[id];
+                keep = may_reach(co.x, co.y, co.z, (float)x0 + 0.5f - xy.x, (float)(x0 + LX) - 0.5f - xy.x,
+                                 (float)y0 + 0.5f - xy.y, (float)(y0 + BH) - 0.5f - xy.y, qmax);
+            }
+            const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+            const int n = __popc(kept);
+            if (keep) {
+                const int slot = __popc(kept & ((1u << lane) - 1u));
+                sm.a[slot] = make_float4(xy.x, xy.y, co.x, 2.0f * co.y);
+                sm.b[slot] = make_float4(co.z, co.w, rgb[3 * (size_t)id], rgb[3 * (size_t)id + 1]);
+                sm.c[slot] = rgb[3 * (size_t)id + 2];
+                sm.pos[slot] = pos;
+            }
+            __syncwarp();
+            auto walk = [&](int j, auto masked) {
+                const float4 ra = sm.a[j], rb = sm.b[j];
+                const float rc = sm.c[j];
+                const int rpos = sm.pos[j];
+                const float dx1 = __fsub_rn(ra.x, fpx);
+                const float2 dx = dup(dx1), y = dup(ra.y), A = dup(ra.z), B2 = dup(ra.w), Cc = dup(rb.x), o = dup(rb.y);
+                const float2 c0 = dup(rb.z), c1 = dup(rb.w), c2 = dup(rc);
+                float2 S0 = dup(0.0f), S1 = dup(0.0f), S2 = dup(0.0f), SF = dup(0.0f), W0 = dup(0.0f), W1 = dup(0.0f),
+                       W2 = dup(0.0f);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    const float2 dy = __fadd2_rn(y, nfpy[v]);
+                    const float2 e = __ffma2_rn(A, dx, __fmul2_rn(B2, dy));  // conic_q
+                    const float2 qr = __ffma2_rn(dx, e, __fmul2_rn(__fmul2_rn(Cc, dy), dy));
+                    // outside the support the profile is taken at its limit: finite, so that the pair's zero
+                    // weight leaves the sums alone (as unsigned words negative values lie above the limit too)
+                    const uint32_t q0 = __float_as_uint(qr.x), q1 = __float_as_uint(qr.y);
+                    const float2 q = make_float2(__uint_as_float(min(q0, qlim)), __uint_as_float(min(q1, qlim)));
+                    float2 F, dF;
+                    if constexpr (KIND == DARB_GENERIC) {  // costly: skipped where no lane is in the support
+                        F = dF = dup(0.0f);
+                        if (__any_sync(0xffffffffu, q0 <= qlim || q1 <= qlim)) {
+                            generic_both(q.x, ks, F.x, dF.x);
+                            generic_both(q.y, ks, F.y, dF.y);
+                        }
+                    } else {
+                        F = kernel_F_lanes<KIND, 2>(q, ks);
+                        dF = kernel_dF2<KIND>(q, F);
                     }
-                } else {
-                    F = kernel_F_lanes<KIND, 2>(q, ks);
-                    dF = kernel_dF2<KIND>(q, F);
+                    const float2 of = __fmul2_rn(o, F);
+                    const float al0 = fminf(kAlphaMax, of.x), al1 = fminf(kAlphaMax, of.y);
+                    const bool u0 = rpos < my_last[2 * v] && q0 <= qlim && al0 >= kAlphaMin;
+                    const bool u1 = rpos < my_last[2 * v + 1] && q1 <= qlim && al1 >= kAlphaMin;
+                    const float2 a = make_float2(u0 ? al0 : 0.0f, u1 ? al1 : 0.0f);
+                    const float2 om = __ffma2_rn(a, dup(-1.0f), dup(1.0f));
+                    const float2 iom = make_float2(rcp_ftz(om.x), rcp_ftz(om.y));
+                    const float2 Tk = __fmul2_rn(T[v], iom);
+                    float2 h0 = g0[v], h1 = g1[v], h2 = g2[v];
+                    if constexpr (decltype(masked)::value) {
+                        if (!u0) h0.x = h1.x = h2.x = 0.0f;
+                        if (!u1) h0.y = h1.y = h2.y = 0.0f;
+                    }
+                    const float2 gc = __ffma2_rn(h2, c2, __ffma2_rn(h1, c1, __fmul2_rn(h0, c0)));
+                    const float2 dal = __ffma2_rn(Tk, gc, __fmul2_rn(__fmul2_rn(GS[v], dup(-1.0f)), iom));
+                    const float2 w = __fmul2_rn(a, Tk);
+                    GS[v] = __ffma2_rn(gc, w, GS[v]);
+                    T[v] = Tk;
+                    W0 = __ffma2_rn(w, h0, W0);
+                    W1 = __ffma2_rn(w, h1, W1);
+                    W2 = __ffma2_rn(w, h2, W2);
+                    // the alpha clamp has zero derivative
+                    const float2 da = make_float2(u0 && !(of.x > kAlphaMax) ? dal.x : 0.0f,
+                                                  u1 && !(of.y > kAlphaMax) ? dal.y : 0.0f);
+                    SF = __ffma2_rn(F, da, SF);
+                    const float2 sq = __fmul2_rn(dF, da);
+                    const float2 p = __fmul2_rn(sq, dy);
+                    S0 = __fadd2_rn(S0, sq);
+                    S1 = __fadd2_rn(S1, p);
+                    S2 = __ffma2_rn(p, dy, S2);
                 }
-                const float2 of = __fmul2_rn(o, F);
-                const float al0 = fminf(kAlphaMax, of.x), al1 = fminf(kAlphaMax, of.y);
-                const bool u0 = rpos < my_last[2 * v] && q0 <= qlim && al0 >= kAlphaMin;
-                const bool u1 = rpos < my_last[2 * v + 1] && q1 <= qlim && al1 >= kAlphaMin;
-                const float2 a = make_float2(u0 ? al0 : 0.0f, u1 ? al1 : 0.0f);
-                const float2 om = __ffma2_rn(a, dup(-1.0f), dup(1.0f));
-                const float2 iom = make_float2(rcp_ftz(om.x), rcp_ftz(om.y));
-                const float2 Tk = __fmul2_rn(T[v], iom);
-                float2 h0 = g0[v], h1 = g1[v], h2 = g2[v];
-                if constexpr (decltype(masked)::value) {
-                    if (!u0) h0.x = h1.x = h2.x = 0.0f;
-                    if (!u1) h0.y = h1.y = h2.y = 0.0f;
+                const float t0 = S0.x + S0.y, t1 = S1.x + S1.y, m0 = t0 * dx1;
+                const float sums[9] = {m0, t1, m0 * dx1, t1 * dx1, S2.x + S2.y, SF.x + SF.y, W0.x + W0.y, W1.x + W1.y,
+                                       W2.x + W2.y};
+                float r8;
+                float r = warp_sum8(sums, lane, r8);
+                // lanes 0, 4, .. 28 hold the first eight sums, every lane the ninth: lane 1 takes that
+                r = lane == 1 ? r8 : r;
+                if ((lane & 3) == 0 || lane == 1) {
+                    const int u = lane == 1 ? 8 : lane >> 2;
+                    sm.sum[9 * (rpos - win) + u] += r;
                 }
-                const float2 gc = __ffma2_rn(h2, c2, __ffma2_rn(h1, c1, __fmul2_rn(h0, c0)));
-                const float2 dal = __ffma2_rn(Tk, gc, __fmul2_rn(__fmul2_rn(GS[v], dup(-1.0f)), iom));
-                const float2 w = __fmul2_rn(a, Tk);
-                GS[v] = __ffma2_rn(gc, w, GS[v]);
-                T[v] = Tk;
-                W0 = __ffma2_rn(w, h0, W0);
-                W1 = __ffma2_rn(w, h1, W1);
-                W2 = __ffma2_rn(w, h2, W2);
-                // the alpha clamp has zero derivative
-                const float2 da = make_float2(u0 && !(of.x > kAlphaMax) ? dal.x : 0.0f,
-                                              u1 && !(of.y > kAlphaMax) ? dal.y : 0.0f);
-                SF = __ffma2_rn(F, da, SF);
-                const float2 sq = __fmul2_rn(dF, da);
-                const float2 p = __fmul2_rn(sq, dy);
-                S0 = __fadd2_rn(S0, sq);
-                S1 = __fadd2_rn(S1, p);
-                S2 = __ffma2_rn(p, dy, S2);
-            }
-            const float t0 = S0.x + S0.y, t1 = S1.x + S1.y, m0 = t0 * dx1;
-            const float sums[9] = {m0, t1, m0 * dx1, t1 * dx1, S2.x + S2.y, SF.x + SF.y, W0.x + W0.y, W1.x + W1.y,
-                                   W2.x + W2.y};
-            float r8;
-            const float r = warp_sum8(sums, lane, r8);
-            if ((lane & 3) == 0) s_sum[j][lane >> 2] = r;
-            if (lane == 1) s_sum[j][8] = r8;
-        };
-        if (odd)
-            for (int j = 0; j < n; ++j) walk(j, std::true_type{});
-        else
-            for (int j = 0; j < n; ++j) walk(j, std::false_type{});
-        __syncwarp();
-        if (lane < n) {
-            const float *s = s_sum[lane];
-            bool any = false;
-#pragma unroll
-            for (int u = 0; u < 9; ++u) any |= s[u] != 0.0f;
-            if (any) {
-                const float4 ra = s_a[lane], rb = s_b[lane];
-                const float A = ra.z, B = 0.5f * ra.w, C = rb.x, o = rb.y;
-                float4 *gp = grad2d + 3 * (size_t)s_id[lane];
-                atomicAdd(gp, make_float4(2.0f * o * (A * s[0] + B * s[1]), 2.0f * o * (B * s[0] + C * s[1]), o * s[2],
-                                          2.0f * o * s[3]));
-                atomicAdd(gp + 1, make_float4(o * s[4], s[5], s[6], s[7]));
-                atomicAdd(reinterpret_cast<float *>(gp + 2), s[8]);
-            }
+            };
+            if (odd)
+                for (int j = 0; j < n; ++j) walk(j, std::true_type{});
+            else
+                for (int j = 0; j < n; ++j) walk(j, std::false_type{});
+            __syncwarp();
         }
-        __syncwarp();
+        __syncthreads();
+        for (int i = threadIdx.x; i < end; i += 32 * NW) {
+            float s[9];
+#pragma unroll
+            for (int u = 0; u < 9; ++u) s[u] = 0.0f;
+#pragma unroll
+            for (int w = 0; w < NW; ++w)
+#pragma unroll
+                for (int u = 0; u < 9; ++u) s[u] += smem[w].sum[9 * i + u];
+            const uint32_t id = values[start + win + i];
+            emit(id, conic_o[id], s);
+        }
+        if (win > 0) __syncthreads();
     }
 }
 
@@ -718,14 +747,14 @@ cudaError_t fwd_t(int n_tiles, const uint2 *ranges, const uint32_t *values, cons
     return cudaGetLastError();
 }
 
-template <int KIND, int LX, int PIX>
+template <int KIND, int TILE, int LX, int PIX>
 cudaError_t bwd_t(int n_tiles, const uint2 *ranges, const uint32_t *values, const float2 *mean2d,
-                  const float4 *conic_o, const float *rgb, const Cam &cam, int tiles_x, int tile, float qmax, int strict,
+                  const float4 *conic_o, const float *rgb, const Cam &cam, int tiles_x, float qmax, int strict,
                   const KernelSpec &ks, const float *t_final, const uint32_t *last, const float *dL, float *grad2d,
                   cudaStream_t st) {
-    const int parts = (tile / LX) * (tile / (32 / LX * PIX));
-    launch_k(k_render_bwd<KIND, LX, PIX>, n_tiles * parts, 32, 0, st,
-             ranges, values, mean2d, conic_o, rgb, cam.W, cam.H, tiles_x, tile, qmax, strict, ks,
+    constexpr int NW = TILE / LX * (TILE / (32 / LX * PIX));
+    launch_k(k_render_bwd<KIND, LX, PIX, NW>, n_tiles, 32 * NW, 0, st,
+             ranges, values, mean2d, conic_o, rgb, cam.W, cam.H, tiles_x, TILE, qmax, strict, ks,
              Bg{cam.bg[0], cam.bg[1], cam.bg[2]}, t_final, last, dL, reinterpret_cast<float4 *>(grad2d));
     return cudaGetLastError();
 }
@@ -841,13 +870,16 @@ cudaError_t launch_render_bwd(int kind, int tile, int tiles_x, int tiles_y, cons
     const int n_tiles = tiles_x * tiles_y;
     if (n_tiles == 0) return cudaSuccess;
     const uint2 *rg = reinterpret_cast<const uint2 *>(ranges);
-    // 16 x 8 blocks (four pixels a lane), but 16 x 4 where the image has fewer than 26 blocks of 16 x 8 per
-    // SM: the chip is then not full, and a warp's time is its own chain.  Measured (sinc, 300k and 20k
-    // splats): 480 x 270 69 -> 56 us, 640 x 360 63 -> 58 and 54 -> 44, 800 x 450 74 -> 67; at 960 x 540 (27
-    // blocks per SM) 78 either way and 62 -> 59; at 1245 x 825 113 -> 126.
-    const bool few = (long long)n_tiles * (tile * tile / 128) < 26ll * kGridSms;
-#define BWD_ARGS n_tiles, rg, values, mean2d, conic_o, rgb, cam, tiles_x, tile, qmax, strict, ks, t_final, last, dL_dimage, grad2d, st
-#define BWD_CALL(K) (tile == 8 ? bwd_t<K, 8, 2>(BWD_ARGS) : few ? bwd_t<K, 16, 2>(BWD_ARGS) : bwd_t<K, 16, 4>(BWD_ARGS))
+    // 16 x 8 blocks (four pixels a lane), but 16 x 4 in 16-pixel tiles where the image has fewer than 48
+    // blocks of 16 x 8 per SM: the chip is then not full, and a warp's time is its own chain.  Measured
+    // (sinc, 20k and 300k splats): 333 x 207 115 -> 67 and 132 -> 79 us, 640 x 360 72 -> 47 and 84 -> 63, 960 x
+    // 540 70 -> 57 and 86 -> 78, 1280 x 720 (47 blocks per SM) 77 -> 71 and 112 -> 112; 1245 x 825 (54)
+    // 84 -> 77 and 122 -> 124, 1080p 120 -> 120 and 194 -> 210.  In 32-pixel tiles the CTAs of sixteen warps
+    // that 16 x 4 blocks need were slower at every size (333 x 207: 148 -> 163, 960 x 540: 86 -> 109).
+    const bool few = (long long)n_tiles * (tile * tile / 128) < 48ll * kGridSms;
+#define BWD_ARGS n_tiles, rg, values, mean2d, conic_o, rgb, cam, tiles_x, qmax, strict, ks, t_final, last, dL_dimage, grad2d, st
+#define BWD_CALL(K) (tile == 8 ? bwd_t<K, 8, 8, 2>(BWD_ARGS) : tile == 32 ? bwd_t<K, 32, 16, 4>(BWD_ARGS) \
+                     : few ? bwd_t<K, 16, 16, 2>(BWD_ARGS) : bwd_t<K, 16, 16, 4>(BWD_ARGS))
     switch (kind) {
     case 0: return BWD_CALL(0); case 1: return BWD_CALL(1); case 2: return BWD_CALL(2); case 3: return BWD_CALL(3);
     case 4: return BWD_CALL(4); case 5: return BWD_CALL(5); case 6: return BWD_CALL(6); default: return BWD_CALL(7);

@@ -74,6 +74,33 @@ def test_compositing_backward_on_either_side_of_its_block_rule(kernel, tile, wid
         grad_close(f"grad2d[{u}]", to_np(got)[:, u], np.asarray(g2)[:, u])
 
 
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("n", [96, 97, 128, 129, 300])
+def test_compositing_backward_at_the_edges_of_its_windows(n, tile):
+    """Faint splats that all cover the image, so that every pixel's run is as long as the list: windows are
+    of 96 records (32-pixel tiles) and 128."""
+    s = synth.uniform_cube_scene(n, seed=5, half=0.3, log_scale=(-0.5, 0.5))
+    s.opacities[:] = np.linspace(0.008, 0.016, n, dtype=np.float32)
+    cam = synth.pinhole((0.5, 0.4, 6.0), 40, 33, 60.0, bg=(0.2, 0.1, 0.4))
+    r, sd, proj, bins, img = gpu_forward(s, cam, "gaussian", tile)
+    ref = oracle.forward(s, cam, "gaussian", tile=tile)
+    check_render(img, bins, ref, cam, tile)
+    assert int(img.n_contrib.max()) > 0.9 * n
+    dl = ambiguity_masked_grad(synth.random_image_grad(33, 40, seed=4), ref["amb"])
+    _, g2, _ = oracle.gradients(s, cam, dl, "gaussian", tile=tile)
+    got = darb.darb_render_bwd(proj, s.n, bins, cam, r.kparams, tile, img, _t(dl.astype(np.float32)))
+    torch.cuda.synchronize()
+    for u in range(9):
+        grad_close(f"grad2d[{u}]", to_np(got)[:, u], np.asarray(g2)[:, u])
+
+
+@pytest.mark.parametrize("kernel", ["gaussian", "mod_sinc"])
+@pytest.mark.parametrize("width,height", [(960, 544), (1280, 720), (1312, 720)])
+def test_compositing_backward_block_rule_of_16_pixel_tiles(kernel, width, height):
+    """Fewer than 7296 blocks of 16 x 8 pixels take two pixels a lane: 4080, 7200 and 7380 blocks."""
+    test_compositing_backward_on_either_side_of_its_block_rule(kernel, 16, width, height)
+
+
 @pytest.mark.parametrize("bad", [np.inf, np.nan])
 def test_gradient_that_is_not_finite_stays_with_the_splats_its_pixel_blended(bad):
     s = synth.cluster_scene(4000, seed=8, sh_degree=0)
