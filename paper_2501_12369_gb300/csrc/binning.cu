@@ -26,6 +26,8 @@
 //                                         (p = 2 at 1080p with 16- or 32-pixel tiles); the last
 //                                         writes only the values
 //   k_keys64 (optional)                   the 64-bit keys, when the caller asks for them
+//   Up to 32768 splats k_small_depth_sort, one cluster, takes the place of the compaction, the depth
+//   passes and the offsets; k_tile_diff then reads all splats.
 //   About 20 bytes of HBM traffic per instance at p = 2.  (With the reduce-then-scan passes,
 //   k_duplicate_balanced writes the instances and the first pass reads them back.)
 //
