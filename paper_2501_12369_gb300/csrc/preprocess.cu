@@ -265,7 +265,7 @@ struct PreGeom {
     int radius, idx;
 };
 
-// Compiled for 9 resident CTAs per SM (48 registers, 1152 threads, each with DARB_PRE_SPT = 2
+// Compiled for 9 resident CTAs per SM (56 registers, 1152 threads, each with DARB_PRE_SPT = 2
 // splats): the projection is latency-bound.  Small CTAs end sooner once their queue, some 40% of the
 // splats, no longer fills every warp: 1M splats, 1080p, 32-pixel tiles (16-pixel; 3M splats): 54.6
 // (71.6; 136) us with 5 CTAs of 256 threads, 52.5 (68.8; 130) with 10 of 128, 51.7 (68.7; 129) with 9,
@@ -285,26 +285,70 @@ struct PreGeom {
 #define DARB_PRE_BOUNDS __launch_bounds__(kPreThreads)
 #endif
 
-// Phase 2 of k_preprocess for one queued (projected, not culled) splat: member tiles by row
-// runs, the records, the SH colour.
+// Phase 2 of k_preprocess for a warp's queued (projected, not culled) splats, a splat a lane: member
+// tiles by row runs, the records, the SH colour.  A few near splats with tall rectangles held up their
+// whole warps, so once a row of the lanes that still have some costs more than handing each of their
+// splats to the warp, a row a lane (about two rows' time), the warp takes them one after the other;
+// at the earliest after the rows that a packed word holds.  1M splats, 1080p, tiles of 32 / 16 / 8:
+// 51.9 / 69.2 / 106 -> 48.3 / 54.3 / 72.9 us; 3M 129 -> 125.5.  Always from the ninth row on 48.3 / 63.5 / 99.5
+// (with the splat's constants computed again by every lane), where a splat counts one row 48.2 / 55.1 / 77.3, where
+// it counts five 49.0 / 55.7 / 72.3.
 template <int DEG>
-__device__ __forceinline__ void preprocess_queued(const PreGeom &g, const float *__restrict__ means,
+__device__ __forceinline__ void preprocess_queued(const PreGeom *q, int e, int nq, const float *__restrict__ means,
                                                   const float *__restrict__ opac, const float *__restrict__ sh,
                                                   const Cam &cam, int tile, float qmax, const ProjectedOut &out) {
+    const int lane = threadIdx.x & 31;
+    const bool mine = e < nq;
+    const PreGeom &g = q[mine ? e : nq - 1];
     const int i = g.idx;
     const SpanCtx sc = make_span_ctx(qmax, tile, cam.W, cam.H);
     const int4 r = make_int4(g.rect[0], g.rect[1], g.rect[2], g.rect[3]);
     uint32_t cnt = 0;  // member tiles: the ellipse's run in every row of the rectangle
     const bool pack = runs_packable(r);
     uint64_t runs = pack ? kRunsNone : kRunsUnpacked;
+    const int rows = mine ? r.w - r.y + 1 : 0, most = (int)__reduce_max_sync(0xffffffffu, (unsigned)rows);
+    int k = 0;
+    uint32_t tall = 0;
     const SpanSplat sp = span_prepare(g.u0, g.u1, g.A, g.B, g.C, qmax);
-    for (int ty = r.y; ty <= r.w; ++ty) {
+    for (; k < most; ++k) {
+        if (k >= kRunsRows) {  // packed runs are whole by then
+            tall = __ballot_sync(0xffffffffu, k < rows);
+            if (2 * __popc(tall) < most - k) break;
+        }
         int c0, c1;
-        if (span_row(sp, sc, r, ty, c0, c1)) {
+        if (k < rows && span_row(sp, sc, r, r.y + k, c0, c1)) {
             cnt += (uint32_t)(c1 - c0 + 1);
-            if (pack) runs = runs_put(runs, r, ty, c0, c1);
+            if (pack) runs = runs_put(runs, r, r.y + k, c0, c1);
         }
     }
+    if (k == most) tall = 0;
+    for (; tall; tall &= tall - 1) {
+        const int l = __ffs(tall) - 1;
+        const PreGeom &t = q[e - lane + l];
+        const int4 tr = make_int4(t.rect[0], t.rect[1], t.rect[2], t.rect[3]);
+        SpanSplat ts;
+        auto of = [&](float v) { return __shfl_sync(0xffffffffu, v, l); };
+        ts.u0 = t.u0;
+        ts.u1 = t.u1;
+        ts.nB = -t.B;
+        ts.det = of(sp.det);
+        ts.ym = of(sp.ym);
+        ts.dyR0 = of(sp.dyR0);
+        ts.dyL0 = -ts.dyR0;
+        ts.aq = of(sp.aq);
+        ts.invA = of(sp.invA);
+        ts.rR = of(sp.rR);
+        ts.rL = -ts.rR;
+        ts.ok = ts.det > 0.0f;
+        uint32_t w = 0;
+        for (int ty = tr.y + k + lane; ty <= tr.w; ty += 32) {
+            int c0, c1;
+            if (span_row(ts, sc, tr, ty, c0, c1)) w += (uint32_t)(c1 - c0 + 1);
+        }
+        w = __reduce_add_sync(0xffffffffu, w);
+        if (lane == l) cnt += w;
+    }
+    if (!mine) return;
     if (cnt == 0) {  // an ellipse that reaches no tile: culled
         write_culled(out, i);
         return;
@@ -409,8 +453,8 @@ k_preprocess(int n, const float *__restrict__ means, const float *__restrict__ s
     }
     __syncthreads();
     const int nq = s_n;
-    for (int e = threadIdx.x; e < nq; e += kPreThreads) preprocess_queued<DEG>(s_q[e], means, opac, sh, cam, tile, qmax,
-                                                                               out);
+    for (int e = threadIdx.x; e - (int)(threadIdx.x & 31) < nq; e += kPreThreads)  // whole warps
+        preprocess_queued<DEG>(s_q, e, nq, means, opac, sh, cam, tile, qmax, out);
 }
 
 

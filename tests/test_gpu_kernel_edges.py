@@ -6,7 +6,7 @@ import torch
 import oracle
 from paper_2501_12369_gb300 import darb, synth
 
-from gpu_helpers import ambiguity_masked_grad, check_lists, check_render, gpu_forward, grad_close, to_np
+from gpu_helpers import ambiguity_masked_grad, check_lists, check_preprocess, check_render, gpu_forward, grad_close, to_np
 from test_gpu_density import CFG, RAW, STATE_OF, _case, _device, _t
 
 pytestmark = [pytest.mark.gpu,
@@ -231,3 +231,18 @@ def test_l1_epilogue_loss_at_cluster_edges(width, height, tile):
     assert abs(float(loss[0]) - np.abs(d).mean()) <= 1.1e-5 * np.abs(d).mean()
     np.testing.assert_array_equal(to_np(out.image), to_np(img.image))
     np.testing.assert_array_equal(to_np(dl), np.sign(d).astype(np.float32) * np.float32(1.0 / (3.0 * width * height)))
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("n", [1, 33, 700])
+def test_member_tiles_of_tall_rectangles(n, tile):
+    """Splats from a pixel to the whole image: rectangles within a packed word's 8 rows, a few taller ones beside
+    them and warps of tall ones, up to 163 rows (more than a warp's lanes)."""
+    s = synth.uniform_cube_scene(n, seed=12, half=1.5, log_scale=(-5.0, 0.7))
+    s.scales[::32] = 1.0
+    cam = synth.pinhole((0.5, 0.4, 6.0), 333, 1300, 600.0, bg=(0.2, 0.1, 0.4))
+    r, sd, proj, bins, img = gpu_forward(s, cam, "gaussian", tile)
+    ref = oracle.project(s, cam, oracle.kernel_params("gaussian"), tile, True)
+    rect = to_np(proj.tile_rect)[0]
+    assert rect[3] - rect[1] + 1 > 8
+    check_preprocess(proj, ref)
