@@ -630,8 +630,10 @@ def run_ours(args):
         "gpu_launches": None,
         "clocks": clk,
     }
-    line["gpu_launches"] = args.steps * launches_per_step(args.sort, int(np.ceil(np.log2(ts.tx * ts.ty))),
-                                                          not args.unfused)
+    # beside those counted there: the launch that folds the conic's sums after the compositing backward
+    # (the unfused Adam is one launch, where five are counted)
+    line["gpu_launches"] = args.steps * (launches_per_step(args.sort, int(np.ceil(np.log2(ts.tx * ts.ty))),
+                                                           not args.unfused) + (-3 if args.unfused else 1))
     line["config"]["optimizer"] = "adam (separate)" if args.unfused else "adam fused into preprocess backward"
     line["config"]["sort"] = "depth_then_tile" if args.sort == 0 else "keys64"
     # the paper's full image loss: (1 - 0.2) L1 + 0.2 D-SSIM in place of L1

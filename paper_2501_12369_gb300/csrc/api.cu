@@ -244,7 +244,7 @@ darb_status darb_render_bwd(const darb_projected *proj, int32_t n, const darb_bi
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (n > 0) DARB_CUDA_TRY(launch_zero(st, grad2d, (size_t)n * 12 * sizeof(float)));
     const int tiles_x = tile_count(cam->width, tile), tiles_y = tile_count(cam->height, tile);
-    DARB_CUDA_TRY(launch_render_bwd(kparams->kind, tile, tiles_x, tiles_y, bins->ranges, bins->values,
+    DARB_CUDA_TRY(launch_render_bwd(kparams->kind, n, proj->tiles_touched, tile, tiles_x, tiles_y, bins->ranges, bins->values,
                                     reinterpret_cast<const float2 *>(proj->mean2d),
                                     reinterpret_cast<const float4 *>(proj->conic_o), proj->rgb, make_cam(*cam),
                                     kparams->q_max, kparams->q_max_strict ? 1 : 0, make_spec(*kparams), fwd->t_final,

@@ -500,6 +500,44 @@ __device__ __forceinline__ bool may_reach(float A, float B, float C, float xl, f
     return !(m > 1.05f * qmax);
 }
 
+// a + b - fl(a + b), exactly (Knuth's two-sum).
+__device__ __forceinline__ float add_error(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// The conic's three sums take up what their additions in memory lost, which k_render_bwd keeps in the
+// last three floats of a row for splats of kManyTiles tiles or more; these are zero again.  Bound by latency
+// (tile counts, rows, stores): 10 us for 3M splats, four a thread (15 with one, 20 for every visible splat).
+// Fewer than kManyTiles additions cost no more than the last rounding of the sum itself.
+constexpr uint32_t kManyTiles = 8;
+__global__ void __launch_bounds__(256)
+k_fold_conic(int n, const uint32_t *__restrict__ tiles, float4 *__restrict__ grad2d) {
+    pdl_entry();
+    const int i0 = 4 * (blockIdx.x * 256 + threadIdx.x);
+    if (i0 >= n) return;
+    uint32_t t[4] = {0, 0, 0, 0};
+    if (i0 + 4 <= n) {
+        const uint4 t4 = *reinterpret_cast<const uint4 *>(tiles + i0);
+        t[0] = t4.x, t[1] = t4.y, t[2] = t4.z, t[3] = t4.w;
+    } else {
+        for (int k = 0; i0 + k < n; ++k) t[k] = tiles[i0 + k];
+    }
+    float4 *row = grad2d + 3 * (size_t)i0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (t[k] < kManyTiles) continue;
+        float *g = reinterpret_cast<float *>(row + 3 * k);
+        const float4 lo = row[3 * k + 2];
+        const float hi[3] = {g[2], g[3], g[4]}, lost[3] = {lo.y, lo.z, lo.w};
+        if (lost[0] == 0.0f && lost[1] == 0.0f && lost[2] == 0.0f) continue;
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            if (isfinite(hi[u])) g[2 + u] = hi[u] + lost[u];  // a sum that is not finite lost nothing
+        row[3 * k + 2] = make_float4(lo.x, 0.0f, 0.0f, 0.0f);
+    }
+}
+
 // Backward: replay each pixel back to front from its last contributor.  With T_k the
 // transmittance in front of splat k and S the colour composited behind it (background
 // included), dC/dalpha_k = c_k T_k - S / (1 - alpha_k) and dC/dc_k = alpha_k T_k.  Only the
@@ -525,17 +563,25 @@ __device__ __forceinline__ bool may_reach(float A, float B, float C, float xl, f
 // block instead took 114 us where this takes 122, but made the error of such sums 2.7 times as
 // large.  Windows of 64 cost 1% more; of 96 in CTAs of eight warps, within 48 KB.
 //
+// The conic's gradients go on to the covariance through -K G K, which cancels by a thin splat's aspect
+// ratio squared, so the rounding of the additions in memory, in whatever order they come, showed in the
+// quaternions' and scales' gradients: two equal steps at 3M splats, 1080p differed by 4e-6 in the second
+// moments (mean over ten views, up to 3e-4).  Each addition of the conic's three therefore returns the sum
+// it met, and what it lost to rounding is added to one of the row's three spare floats, which k_fold_conic puts
+// back: two equal steps then agree to 3e-10.  A step went from 1339 to 1353 us.
+//
 // Bound by the FP32 and ALU pipes of the pair body.  Launch, 300k splats, 1245 x 825, 16-pixel tiles, against
 // a thread per pixel column of the tile with scalar arithmetic and a list of kept records for the
 // whole CTA: sinc 217 -> 122 us, Gaussian 367 -> 225, half-cosine 100 -> 64; sinc with 32-pixel tiles
-// 273 -> 135, 8-pixel 237 -> 120; 20k splats 142 -> 84, at 333 x 207 167 -> 67.
+// 273 -> 135, 8-pixel 237 -> 120; 20k splats 142 -> 84, at 333 x 207 167 -> 67.  (Before the two points above,
+// which take 3% and the second launch's 4 us.)
 template <int KIND, int LX, int PIX, int NW>
 __global__ void __launch_bounds__(32 * NW, (PIX == 2 ? 28 : NW == 8 ? 24 : 20) / NW)
 k_render_bwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ values,
              const float2 *__restrict__ mean2d, const float4 *__restrict__ conic_o,
-             const float *__restrict__ rgb, int W, int H, int tiles_x, int tile, float qmax, int strict, KernelSpec ks,
-             Bg bg, const float *__restrict__ t_final, const uint32_t *__restrict__ last,
-             const float *__restrict__ dL_dimage, float4 *__restrict__ grad2d) {
+             const float *__restrict__ rgb, const uint32_t *__restrict__ tiles, int W, int H, int tiles_x, int tile,
+             float qmax, int strict, KernelSpec ks, Bg bg, const float *__restrict__ t_final,
+             const uint32_t *__restrict__ last, const float *__restrict__ dL_dimage, float4 *__restrict__ grad2d) {
     pdl_entry();
     static_assert(PIX == 2 || PIX == 4, "one or two pairs of pixels a lane");
     constexpr int LY = 32 / LX, BH = LY * PIX, NV = PIX / 2, kWindow = NW == 8 ? 96 : 128;
@@ -553,15 +599,22 @@ k_render_bwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ valu
     const uint32_t qlim = __float_as_uint(support_limit(qmax, strict));
     const size_t plane = (size_t)W * H;
     auto dup = [](float a) { return make_float2(a, a); };
-    auto emit = [&](uint32_t id, float o, const float (&s)[9]) {  // a record's sums to its gradients
+    auto emit = [&](uint32_t id, float o, bool many, const float (&s)[9]) {  // a record's sums to its gradients
         bool any = false;
 #pragma unroll
         for (int u = 0; u < 9; ++u) any |= s[u] != 0.0f;
         if (!any) return;
         float4 *gp = grad2d + 3 * (size_t)id;
-        atomicAdd(gp, make_float4(2.0f * o * s[0], 2.0f * o * s[1], o * s[2], 2.0f * o * s[3]));
-        atomicAdd(gp + 1, make_float4(o * s[4], s[5], s[6], s[7]));
-        atomicAdd(reinterpret_cast<float *>(gp + 2), s[8]);
+        const float4 x = make_float4(2.0f * o * s[0], 2.0f * o * s[1], o * s[2], 2.0f * o * s[3]);
+        const float4 y = make_float4(o * s[4], s[5], s[6], s[7]);
+        if (many) {
+            const float4 p = atomicAdd(gp, x), q = atomicAdd(gp + 1, y);
+            atomicAdd(gp + 2, make_float4(s[8], add_error(p.z, x.z), add_error(p.w, x.w), add_error(q.x, y.x)));
+        } else {
+            atomicAdd(gp, x);
+            atomicAdd(gp + 1, y);
+            atomicAdd(reinterpret_cast<float *>(gp + 2), s[8]);
+        }
     };
     const int x0 = (t % tiles_x) * tile + warp % (tile / LX) * LX, y0 = (t / tiles_x) * tile + warp / (tile / LX) * BH;
     const int px = x0 + lane % LX;
@@ -735,7 +788,7 @@ k_render_bwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ valu
 #pragma unroll
                 for (int u = 0; u < 9; ++u) s[u] += smem[w].sum[9 * i + u];
             const uint32_t id = values[start + win + i];
-            emit(id, conic_o[id].w, s);
+            emit(id, conic_o[id].w, tiles[id] >= kManyTiles, s);
         }
         if (win > 0) __syncthreads();
     }
@@ -762,12 +815,12 @@ cudaError_t fwd_t(int n_tiles, const uint2 *ranges, const uint32_t *values, cons
 
 template <int KIND, int TILE, int LX, int PIX>
 cudaError_t bwd_t(int n_tiles, const uint2 *ranges, const uint32_t *values, const float2 *mean2d,
-                  const float4 *conic_o, const float *rgb, const Cam &cam, int tiles_x, float qmax, int strict,
-                  const KernelSpec &ks, const float *t_final, const uint32_t *last, const float *dL, float *grad2d,
+                  const float4 *conic_o, const float *rgb, const uint32_t *tiles, const Cam &cam, int tiles_x, float qmax,
+                  int strict, const KernelSpec &ks, const float *t_final, const uint32_t *last, const float *dL, float *grad2d,
                   cudaStream_t st) {
     constexpr int NW = TILE / LX * (TILE / (32 / LX * PIX));
     launch_k(k_render_bwd<KIND, LX, PIX, NW>, n_tiles, 32 * NW, 0, st,
-             ranges, values, mean2d, conic_o, rgb, cam.W, cam.H, tiles_x, TILE, qmax, strict, ks,
+             ranges, values, mean2d, conic_o, rgb, tiles, cam.W, cam.H, tiles_x, TILE, qmax, strict, ks,
              Bg{cam.bg[0], cam.bg[1], cam.bg[2]}, t_final, last, dL, reinterpret_cast<float4 *>(grad2d));
     return cudaGetLastError();
 }
@@ -875,7 +928,7 @@ cudaError_t launch_render_fwd_batch(int kind, int tile, const BatchView *views, 
 #undef FB_CALL
 }
 
-cudaError_t launch_render_bwd(int kind, int tile, int tiles_x, int tiles_y, const uint32_t *ranges,
+cudaError_t launch_render_bwd(int kind, int n, const uint32_t *tiles, int tile, int tiles_x, int tiles_y, const uint32_t *ranges,
                               const uint32_t *values, const float2 *mean2d, const float4 *conic_o,
                               const float *rgb, const Cam &cam, float qmax, int strict, const KernelSpec &ks,
                               const float *t_final, const uint32_t *last, const float *dL_dimage,
@@ -890,13 +943,17 @@ cudaError_t launch_render_bwd(int kind, int tile, int tiles_x, int tiles_y, cons
     // 84 -> 77 and 122 -> 124, 1080p 120 -> 120 and 194 -> 210.  In 32-pixel tiles the CTAs of sixteen warps
     // that 16 x 4 blocks need were slower at every size (333 x 207: 148 -> 163, 960 x 540: 86 -> 109).
     const bool few = (long long)n_tiles * (tile * tile / 128) < 48ll * kGridSms;
-#define BWD_ARGS n_tiles, rg, values, mean2d, conic_o, rgb, cam, tiles_x, qmax, strict, ks, t_final, last, dL_dimage, grad2d, st
+#define BWD_ARGS n_tiles, rg, values, mean2d, conic_o, rgb, tiles, cam, tiles_x, qmax, strict, ks, t_final, last, dL_dimage, grad2d, st
 #define BWD_CALL(K) (tile == 8 ? bwd_t<K, 8, 8, 2>(BWD_ARGS) : tile == 32 ? bwd_t<K, 32, 16, 4>(BWD_ARGS) \
                      : few ? bwd_t<K, 16, 16, 2>(BWD_ARGS) : bwd_t<K, 16, 16, 4>(BWD_ARGS))
+    cudaError_t e;
     switch (kind) {
-    case 0: return BWD_CALL(0); case 1: return BWD_CALL(1); case 2: return BWD_CALL(2); case 3: return BWD_CALL(3);
-    case 4: return BWD_CALL(4); case 5: return BWD_CALL(5); case 6: return BWD_CALL(6); default: return BWD_CALL(7);
+    case 0: e = BWD_CALL(0); break; case 1: e = BWD_CALL(1); break; case 2: e = BWD_CALL(2); break; case 3: e = BWD_CALL(3); break;
+    case 4: e = BWD_CALL(4); break; case 5: e = BWD_CALL(5); break; case 6: e = BWD_CALL(6); break; default: e = BWD_CALL(7);
     }
+    if (e != cudaSuccess || n == 0 || !tiles) return e;
+    launch_k(k_fold_conic, (n + 1023) / 1024, 256, 0, st, n, tiles, reinterpret_cast<float4 *>(grad2d));
+    return cudaGetLastError();
 #undef BWD_CALL
 #undef BWD_ARGS
 }

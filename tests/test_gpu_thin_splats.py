@@ -76,3 +76,22 @@ def test_centre_gradient_of_thin_splats(length, aspect, tilt, tile):
         got = to_np(darb.darb_render_bwd(proj, 1, bins, cam, r.kparams, tile, img, torch.from_numpy(dl).cuda()))[0]
         errors += [(got[k] - ref) / sigma for k, (ref, sigma) in enumerate(centre_gradient(proj, cam, dl))]
     assert np.sqrt(np.mean(np.square(errors))) <= 2.0, errors
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("length,aspect,tilt", [(900, 2, 0.6), (2400, 3, 0.9)])
+def test_conic_gradients_do_not_depend_on_the_order_of_the_tiles(length, aspect, tilt, tile):
+    """A splat over most of the image and one-signed upstream gradients: the tiles' sums of s dx^2 and s dy^2 all
+    have one sign and that of s dx dy is at most their geometric mean.  With the rounding of every addition kept, a
+    result is off by its own last rounding, so that two agree to 2 U; what the additions of up to 5000 lost
+    parts lose themselves is some 5000 U^2, below U / 1000."""
+    scene, cam = _thin_splat(length, aspect, tilt)
+    r, sd, proj, bins, img = gpu_forward(scene, cam, "gaussian", tile)
+    dl = np.random.default_rng(3).uniform(0.5, 1.5, (3, cam.height, cam.width)).astype(np.float32)
+    dl = torch.from_numpy(dl).cuda()
+    got = np.stack([to_np(darb.darb_render_bwd(proj, 1, bins, cam, r.kparams, tile, img, dl))[0] for _ in range(24)])
+    assert (got[:, 9:] == 0).all()
+    a, b, c = (got[:, k].astype(np.float64) for k in (2, 3, 4))
+    for v, size in ((a, np.abs(a).max()), (c, np.abs(c).max())):
+        assert np.ptp(v) <= 2.01 * U * size
+    assert np.ptp(b) <= 2 * U * np.abs(b).max() + 0.01 * U * np.sqrt(np.abs(a).max() * np.abs(c).max())
