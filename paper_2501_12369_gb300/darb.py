@@ -585,7 +585,7 @@ class Rasterizer:
             self.kparams.psi = float(psi)
         self.device = device
         self.tiles_x, self.tiles_y = darb_tile_grid(cam, tile)
-        self._size = (cam.width, cam.height)
+        self._size = (cam.width, cam.height, self.tile)
         self.capacity = int(capacity) if capacity else 0
         self._ws = None
         self._bins = None
@@ -600,10 +600,11 @@ class Rasterizer:
             self._n = n
 
     def _sort(self, proj, n, owned):
-        if (self.cam.width, self.cam.height) != self._size:
+        size = (self.cam.width, self.cam.height, self.tile)
+        if size != self._size:
             tx, ty = darb_tile_grid(self.cam, self.tile)
-            self._size = (self.cam.width, self.cam.height)
-            if (tx, ty) != (self.tiles_x, self.tiles_y):  # the camera was changed to another resolution
+            self._size = size
+            if (tx, ty) != (self.tiles_x, self.tiles_y):  # another resolution or tile
                 self.tiles_x, self.tiles_y = tx, ty
                 self._ws = None
         self._ensure(n, self.capacity)
