@@ -1864,11 +1864,12 @@ size_t sort_workspace_bytes(int n, uint64_t capacity, int tiles_x, int tiles_y, 
 
 namespace {
 // The side stream of a device that takes the per-tile counts beside the depth passes, and its
-// fork / join events; created on first use, kept for the process.
+// fork / join events; created on first use, kept for the process.  reader takes the copies of M that a
+// synchronous call waits for: s also holds tile counts that other streams' sorts have yet to reach.
 struct SortSide {
     std::mutex mu;
     bool ready = false;
-    cudaStream_t s = nullptr;
+    cudaStream_t s = nullptr, reader = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr, counted = nullptr;
 };
 constexpr int kMaxDevicesSort = 64;
@@ -1877,6 +1878,7 @@ SortSide g_sort_side[kMaxDevicesSort];
 cudaError_t sort_side_init(SortSide &P) {
     if (P.ready) return cudaSuccess;
     cudaError_t e = cudaStreamCreateWithFlags(&P.s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P.reader, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P.fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P.join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P.counted, cudaEventDisableTiming);
@@ -2123,7 +2125,7 @@ cudaError_t launch_bin_sort(int n, const ProjectedIn &proj, int tiles_x, int til
     }
     TRY(cudaGetLastError());
     uint64_t grid = capacity;
-    // A synchronous call reads M on the side stream while the rest of the sort, sized by the capacity, is
+    // A synchronous call reads M on a stream of its own while the rest of the sort, sized by the capacity, is
     // already enqueued: the device then works on while the host wakes up and prepares the compositing,
     // where it stood idle until the host had sized and launched the rest (forward views: 20k splats,
     // 720p 223 -> 207 us, 500k 265 -> 256, 900k 286 -> 275).  Above four
@@ -2225,8 +2227,8 @@ cudaError_t launch_bin_sort(int n, const ProjectedIn &proj, int tiles_x, int til
         TRY(cudaGetLastError());
     }
     if (early) {
-        TRY(cudaStreamWaitEvent(side->s, side->counted, 0));
-        TRY(read_count(side->s));
+        TRY(cudaStreamWaitEvent(side->reader, side->counted, 0));
+        TRY(read_count(side->reader));
     }
     return cudaSuccess;
 #undef TRY
