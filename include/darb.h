@@ -221,8 +221,8 @@ darb_status darb_bin_sort_workspace_size(int32_t n, int32_t tile, const darb_cam
  * darb_bin_sort_workspace_size bytes, contents scratch.  capacity: entries of
  * out->keys / out->values (< 2^30).  num_instances_host: if non-NULL the call waits
  * once, until the stream has counted M, to read it and returns DARB_ERR_CAPACITY when
- * M > capacity (outputs then undefined); if NULL nothing synchronises, the sort is
- * sized by capacity, and an overflow is reported in out->status with every tile range
+ * M > capacity (outputs then undefined, and nothing of the call in flight on the stream any
+ * more); if NULL nothing synchronises, the sort is sized by capacity, and an overflow is reported in out->status with every tile range
  * left empty (so a following darb_render_fwd draws only the background).  The per-tile counts
  * run on a side stream of the library (one per device, created by the first call, so make one
  * call before capturing the stream), forked from and joined back to `stream` with events,

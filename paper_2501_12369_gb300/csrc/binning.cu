@@ -2141,9 +2141,16 @@ cudaError_t launch_bin_sort(int n, const ProjectedIn &proj, int tiles_x, int til
         *capacity_exceeded = M > capacity;
         return cudaSuccess;
     };
+    // After an overflow nothing of the call is left in flight: the caller may free its buffers at once, or
+    // sort into them on another stream.
+    auto drain = [&] {
+        TRY(side_join.join());
+        if (side_lock.owns_lock()) side_lock.unlock();
+        return cudaStreamSynchronize(st);
+    };
     if (num_instances_host && !early) {
         TRY(read_count(st));
-        if (*capacity_exceeded) return cudaSuccess;
+        if (*capacity_exceeded) return drain();
         grid = *num_instances_host;
     }
     // 3) per-tile counts from the rectangles -> ranges and tile-pass digit bases (done above
@@ -2229,6 +2236,7 @@ cudaError_t launch_bin_sort(int n, const ProjectedIn &proj, int tiles_x, int til
     if (early) {
         TRY(cudaStreamWaitEvent(side->reader, side->counted, 0));
         TRY(read_count(side->reader));
+        if (*capacity_exceeded) return drain();
     }
     return cudaSuccess;
 #undef TRY

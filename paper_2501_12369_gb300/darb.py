@@ -384,8 +384,10 @@ def darb_bin_sort_workspace_size(n, tile, cam, capacity, strategy=DARB_SORT_DEPT
 
 def darb_bin_sort(proj: Projected, n, tile, cam, workspace: torch.Tensor, capacity, out: Binning | None = None,
                   sync=True, stream=None, strategy=DARB_SORT_DEPTH_THEN_TILE, kparams=None):
-    """sync=True reads M back (one stream synchronisation) and sizes the sort by it.  kparams:
-    the kernel the records were projected with (default: the one darb_preprocess recorded)."""
+    """sync=True waits until the stream has counted M and reads it back; an M above the capacity raises
+    DarbError (with .M) after everything of the call has finished.  The sort itself goes on after the
+    call.  kparams: the kernel the records were projected with (default: the one darb_preprocess
+    recorded)."""
     if out is None:
         tx, ty = darb_tile_grid(cam, tile)
         out = Binning.empty(capacity, tx * ty, workspace.device)

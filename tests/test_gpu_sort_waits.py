@@ -1,4 +1,4 @@
-"""What a synchronous sort waits for."""
+"""What a synchronous sort waits for, and what it leaves in flight."""
 import time
 
 import pytest
@@ -49,3 +49,28 @@ def test_synchronous_sort_does_not_wait_for_another_streams_sort():
     torch.cuda.synchronize()
     assert got == m and pending, f"the synchronous sort returned after {t:.3f} s, with the other stream's"
     assert int(to_np(kept[0].num_instances)[0]) == m
+
+
+@pytest.mark.parametrize("n,capacity", [(2000, 1 << 12), (200000, 1 << 18), (200000, 1)])
+def test_overflow_leaves_nothing_in_flight(n, capacity):
+    """After DARB_ERR_CAPACITY the buffers may be freed, or used on another stream at once.  The tile counts (and with
+    them the rest of the sort) are held up by another stream's."""
+    sort = _view(n)
+    first, _ = sort(1 << 21, True)
+    m = first.M
+    assert m > capacity
+    ref = to_np(first.values)[:m], to_np(first.ranges)
+    other = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(other):
+        torch.cuda._sleep(int(2.0e8))  # a tenth of a second
+        kept = sort(1 << 21, False)
+    with pytest.raises(darb.DarbError) as e:
+        sort(capacity, True)
+    assert torch.cuda.current_stream().query()
+    assert e.value.status == 3 and e.value.M == m
+    with torch.cuda.stream(torch.cuda.Stream()):
+        again, _ = sort(m, True)
+    torch.cuda.synchronize()
+    for b in (again, kept[0]):
+        assert (to_np(b.values)[:m] == ref[0]).all() and (to_np(b.ranges) == ref[1]).all()
