@@ -5,9 +5,9 @@
 // Two kernels over 32 x 32 output tiles of one channel with a 5-pixel halo, both blurs separable in
 // shared memory, every thread 8 consecutive outputs along x and 4 along y (an input is read from
 // shared memory once for all the outputs it reaches):
-//   k_ssim_fwd  stages (x, y) pairs, blurs the four moments that SSIM needs (x, y, x^2 + y^2, xy: s_xx
-//               and s_yy enter B2 only as their sum), and writes per pixel the partial derivatives of
-//               SSIM w.r.t. the local moments m_x, s_xx, s_xy, plus the block sums of SSIM and |x - y|;
+//   k_ssim_fwd  stages (x, y) pairs, blurs the four moments that SSIM needs (x, y, (x - y)^2, xy), and
+//               writes per pixel the partial derivatives of SSIM w.r.t. the local moments m_x, s_xx,
+//               s_xy, plus the block sums of SSIM and |x - y|;
 //   k_ssim_bwd  blurs those three maps (the window is symmetric, so the blur is its own adjoint)
 //               and forms dL/dx = (1 - lambda) sign(x - y) / N - lambda (G*d_m + 2x G*d_sxx +
 //               y G*d_sxy) / N, N = 3HW; its first CTA also writes the loss.
@@ -15,6 +15,10 @@
 // B2 = s_xx - m_x^2 + s_yy - m_y^2 + C2 and SSIM = A1 A2 / (B1 B2):
 //   d_m = 2 m_y (A2 - A1) / (B1 B2) - 2 m_x SSIM (1/B1 - 1/B2),  d_sxx = -SSIM / B2,
 //   d_sxy = 2 A1 / (B1 B2).
+// s_xx and s_yy enter B2 only as their sum, which is the variance of x - y and twice s_xy: B2 = A2 + var(x - y),
+// and B1 = A1 + (m_x - m_y)^2.  What A2 lost to cancellation B2 then shares, and SSIM is near their
+// quotient: on images that are nearly equal the gradient's error against 64 bits is 0.6 to 0.95 of what the five
+// moments gave, where the sum x^2 + y^2 gave 0.9 to 1.24.
 // The forward is bound by issue slots and shared memory (70% and 55% busy), the backward by latency.
 // The quantities blurred under one tap weight lie side by side in shared memory, so they load as the
 // operands of the packed two-lane FMA; columns lie in four planes (column mod 4), which keeps both
@@ -140,7 +144,7 @@ k_ssim_fwd(const float *__restrict__ x, const float *__restrict__ y, int W, int 
            float2 *__restrict__ d_m_sxx, float *__restrict__ d_sxy, double *__restrict__ sums) {
     pdl_entry();
     __shared__ float2 sxy[4 * kInPlane<float2>];
-    __shared__ float4 h[4 * kOutPlane<float4>];  // blurred along x: x, y, x^2 + y^2, xy
+    __shared__ float4 h[4 * kOutPlane<float4>];  // blurred along x: x, y, (x - y)^2, xy
     __shared__ float s_part[2][kSsimThreads / 32];
     const int tiles_x = (W + kSsimTs - 1) / kSsimTs, tiles_y = (H + kSsimTs - 1) / kSsimTs;
     const size_t plane = (size_t)W * H;
@@ -180,7 +184,8 @@ k_ssim_fwd(const float *__restrict__ x, const float *__restrict__ y, int W, int 
 #pragma unroll
         for (int k = 0; k < kRbX + kSsimTaps - 1; ++k) {
             const float2 v = row[(k & 3) * kInPlane<float2> + (k >> 2)];
-            const float2 p = make_float2(fmaf(v.x, v.x, v.y * v.y), v.x * v.y);
+            const float d = v.x - v.y;
+            const float2 p = make_float2(d * d, v.x * v.y);
 #pragma unroll
             for (int i = 0; i < kRbX; ++i)
                 if (k - i >= 0 && k - i < kSsimTaps) {
@@ -216,11 +221,11 @@ k_ssim_fwd(const float *__restrict__ x, const float *__restrict__ y, int W, int 
         const int r = r0 + i, gy = tile.y0 + r, gx = tile.x0 + c;
         if (gx >= W || gy >= H) continue;
         const float mx = m[i].x, my = m[i].y;
-        const float mxy = mx * my, mm = fmaf(mx, mx, my * my);
-        const float A1 = 2.0f * mxy + kSsimC1;
-        const float A2 = 2.0f * (q[i].y - mxy) + kSsimC2;
-        const float B1 = mm + kSsimC1;
-        const float B2 = (q[i].x - mm) + kSsimC2;
+        const float md = mx - my;
+        const float A1 = 2.0f * mx * my + kSsimC1;
+        const float A2 = 2.0f * fmaf(-mx, my, q[i].y) + kSsimC2;
+        const float B1 = fmaf(md, md, A1);
+        const float B2 = fmaf(-md, md, q[i].x) + A2;
         const float iB = __frcp_rn(B1 * B2), iB1 = iB * B2, iB2 = iB * B1;  // one reciprocal for both
         const float sv = A1 * A2 * iB;
         const size_t p = tile.off + (size_t)gy * W + gx;
