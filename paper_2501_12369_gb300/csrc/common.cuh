@@ -259,7 +259,7 @@ __device__ __forceinline__ void generic_both(float q, const KernelSpec &ks, floa
     }
     const float qq = fmaxf(q, 1e-30f);  // one-sided limit at the centre (finite for beta >= 1 on cosines)
     const float uu = q < 1e-30f ? generic_u(qq, ks) : u;
-    dF = generic_base_du(ks.base, uu) * ks.half_beta * __fdividef(uu, qq);
+    dF = generic_base_du(ks.base, uu) * ks.half_beta * (uu / qq);
 }
 
 // ---------------------------------------------------------------------------

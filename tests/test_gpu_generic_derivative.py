@@ -1,0 +1,57 @@
+"""The generic family's derivative where it is exact."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2501_12369_gb300 import darb, synth
+
+from gpu_helpers import to_np
+
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2501_12369_gb300 import build
+    build.build()
+
+
+def test_derivative_of_a_linear_profile_in_the_distance_is_exact():
+    """F = 1 - sqrt(q) / xi at one pixel with dx = m, dy = 0 and the unit conic: q = m^2, and with 1 / xi = m / 2^k
+    u = m^2 / 2^k, so that u / q = 2^-k and dF/dq = -2^-(k + 1) need no rounding.  The gradients of that pixel
+    are then m dF T and (with alpha = F / 2 = 1 - T before the replay) alpha T in red, each rounded once, T
+    the replayed transmittance, 1 but for its own rounding, which is the same in both."""
+    f = np.float32
+    cam = synth.pinhole((0.0, 0.0, 4.0), 8, 8, 8.0)
+    proj = darb.Projected.empty(1, "cuda")
+    bins = darb.Binning.empty(16, 1, "cuda")
+    bins.values.zero_()
+    bins.ranges[:] = torch.tensor([[0, 1]], dtype=torch.int32)
+    img = darb.ImageOut.empty(8, 8, "cuda")
+    img.last.zero_()
+    img.last[0, 0] = 1
+    img.t_final.fill_(1.0)
+    dl = torch.zeros(3, 8, 8, device="cuda")
+    dl[0, 0, 0] = 1.0
+    for name in ("radius", "tiles_touched"):
+        getattr(proj, name).fill_(1)
+    proj.rgb[:] = torch.tensor([[1.0, 0.0, 0.0]])
+    proj.conic_o[:] = torch.tensor([[1.0, 0.0, 1.0, 0.5]])
+    for m in range(3, 259, 2):
+        k = int(np.ceil(2 * np.log2(m))) + 2
+        inv_xi = f(m) * f(2.0) ** -k
+        near = f(1.0) / inv_xi
+        xi = [x for x in (near, np.nextafter(near, f(0)), np.nextafter(near, f(1e9))) if f(1.0) / x == inv_xi]
+        if not xi:  # no FP32 number has this inverse: 26 of the 128
+            continue
+        kp = darb.darb_kernel_generic("parabola", float(xi[0]), 1.0, 1, 1.0)
+        kp.q_max = 1e5
+        alpha = f(0.5) * (f(1.0) - f(m * m) * f(2.0) ** -k)
+        img.t_final[0, 0] = float(f(1.0) - alpha)
+        proj.mean2d[:] = torch.tensor([[0.5 + m, 0.5]])
+        g = to_np(darb.darb_render_bwd(proj, 1, bins, cam, kp, 8, img, dl))[0]
+        near1 = [f(1.0) + f(j) * f(2.0) ** -24 for j in (-4, -3, -2, -1, 0, 2, 4)]
+        replayed = [t for t in near1 if alpha * t == g[6]]
+        assert replayed, (m, g[6], alpha)
+        assert g[0] in [-f(m) * t * f(2.0) ** -(k + 1) for t in replayed], (m, g[0])
