@@ -180,14 +180,6 @@ template <> __device__ __forceinline__ float kernel_F<DARB_HALF_COSINE>(float q,
 template <> __device__ __forceinline__ float kernel_F<DARB_RAISED_COSINE>(float q, const KernelSpec &) {
     return __fmaf_rn(0.5f, __cosf(__fmul_rn(sqrt_newton(q), kPi / 2.5f)), 0.5f);
 }
-__device__ __forceinline__ float raised_cosine_dF(float q) {
-    // -(k/4) sin(k sqrt q) / sqrt q, k = pi/2.5; limit -k^2/4 at q = 0.
-    constexpr float k = kPi / 2.5f;
-    if (q < 1e-6f) return -0.25f * k * k + (k * k * k * k / 24.0f) * q;
-    const float r = sqrt_newton(q), a = rsqrt_ftz(q);
-    const float ir = __fmaf_rn(a, __fmaf_rn(-r, a, 1.0f), a);  // 1 / r, one Newton step from the approximate one
-    return -0.25f * k * __sinf(k * r) * ir;
-}
 
 template <> __device__ __forceinline__ float kernel_F<DARB_MOD_SINC>(float q, const KernelSpec &) {
     // x = pi sqrt(q) / 3, so x^2 = (pi^2 / 9) q; sin(x)/x >= 0 on the main lobe

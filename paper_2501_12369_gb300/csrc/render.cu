@@ -440,8 +440,9 @@ k_render_fwd_batch(const BatchView *__restrict__ views, int n_views, int total_t
 }
 
 // dF/dq of a pair of values, F the profile there.  Where F gives it, from F; the sinc's from the
-// derivative of its series (to u^7, the next term below 1e-8 on the main lobe), which needs no
-// sine, cosine or division and is nearer the derivative than their quotient was.
+// derivative of its series (to u^7, the next term below 1e-8 on the main lobe) and the raised cosine's
+// from the sinc's series, which need no sine, cosine, root or division and are nearer the derivative than their
+// quotient (the raised cosine's to 4e-7 of its value for q <= 4, where __sinf left 1.7e-5).
 template <int KIND>
 __device__ __forceinline__ float2 kernel_dF2(float2 q, float2 F) {
     auto dup = [](float a) { return make_float2(a, a); };
@@ -469,7 +470,19 @@ __device__ __forceinline__ float2 kernel_dF2(float2 q, float2 F) {
     } else if constexpr (KIND == DARB_PARABOLA) {
         return dup(-1.0f / 9.0f);
     } else {
-        return make_float2(raised_cosine_dF(q.x), raised_cosine_dF(q.y));
+        // raised cosine: -(k^2/4) sin(x)/x, x^2 = u = k^2 q, k = pi/2.5, by the series to u^8 / 17! (the next
+        // term is below 1e-8 at x = pi)
+        constexpr float kk = kPi * kPi / 6.25f;
+        const float2 u = __fmul2_rn(q, dup(kk));
+        float2 r = __ffma2_rn(u, dup(1.0f / 355687428096000.0f), dup(-1.0f / 1307674368000.0f));
+        r = __ffma2_rn(r, u, dup(1.0f / 6227020800.0f));
+        r = __ffma2_rn(r, u, dup(-1.0f / 39916800.0f));
+        r = __ffma2_rn(r, u, dup(1.0f / 362880.0f));
+        r = __ffma2_rn(r, u, dup(-1.0f / 5040.0f));
+        r = __ffma2_rn(r, u, dup(1.0f / 120.0f));
+        r = __ffma2_rn(r, u, dup(-1.0f / 6.0f));
+        r = __ffma2_rn(r, u, dup(1.0f));
+        return __fmul2_rn(r, dup(-0.25f * kk));
     }
 }
 
