@@ -439,6 +439,11 @@ k_render_fwd_batch(const BatchView *__restrict__ views, int n_views, int total_t
     }
 }
 
+// The raised cosine with a q_max past its main lobe (q <= 6.25), as a caller may set it: there F rises again,
+// and the derivative's series has ended.
+constexpr int kRaisedCosineWide = kNumKernels;
+constexpr float kRaisedCosineEnd = 6.5f;
+
 // dF/dq of a pair of values, F the profile there.  Where F gives it, from F; the sinc's from the
 // derivative of its series (to u^7, the next term below 1e-8 on the main lobe) and the raised cosine's
 // from the sinc's series, which need no sine, cosine, root or division and are nearer the derivative than their
@@ -469,6 +474,11 @@ __device__ __forceinline__ float2 kernel_dF2(float2 q, float2 F) {
         return __fmul2_rn(__fmul2_rn(F, F), __fmul2_rn(F, dup(-0.5f)));
     } else if constexpr (KIND == DARB_PARABOLA) {
         return dup(-1.0f / 9.0f);
+    } else if constexpr (KIND == kRaisedCosineWide) {
+        constexpr float k = kPi / 2.5f;
+        auto d = [](float v) { return -0.25f * k * __sinf(k * sqrt_newton(v)) / sqrt_newton(v); };
+        const float2 z = __ffma2_rn(q, dup(k * k * k * k / 24.0f), dup(-0.25f * k * k));  // the limit at q = 0
+        return make_float2(q.x < 1e-6f ? z.x : d(q.x), q.y < 1e-6f ? z.y : d(q.y));
     } else {
         // raised cosine: -(k^2/4) sin(x)/x, x^2 = u = k^2 q, k = pi/2.5, by the series to u^8 / 17! (the next
         // term is below 1e-8 at x = pi)
@@ -755,7 +765,7 @@ k_render_bwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ valu
                             generic_both(q.y, ks, F.y, dF.y);
                         }
                     } else {
-                        F = kernel_F_lanes<KIND, 2>(q, ks);
+                        F = kernel_F_lanes<KIND == kRaisedCosineWide ? DARB_RAISED_COSINE : KIND, 2>(q, ks);
                         dF = kernel_dF2<KIND>(q, F);
                     }
                     const float2 of = __fmul2_rn(o, F);
@@ -991,7 +1001,8 @@ cudaError_t launch_render_bwd(int kind, int n, const uint32_t *tiles, int tile, 
                      : few ? bwd_t<K, 16, 16, 2>(BWD_ARGS) : bwd_t<K, 16, 16, 4>(BWD_ARGS))
     cudaError_t e;
     switch (kind) {
-    case 0: e = BWD_CALL(0); break; case 1: e = BWD_CALL(1); break; case 2: e = BWD_CALL(2); break; case 3: e = BWD_CALL(3); break;
+    case 0: e = BWD_CALL(0); break; case 1: e = BWD_CALL(1); break; case 3: e = BWD_CALL(3); break;
+    case DARB_RAISED_COSINE: e = qmax > kRaisedCosineEnd ? BWD_CALL(kRaisedCosineWide) : BWD_CALL(2); break;
     case 4: e = BWD_CALL(4); break; case 5: e = BWD_CALL(5); break; case 6: e = BWD_CALL(6); break; default: e = BWD_CALL(7);
     }
     if (e != cudaSuccess || n == 0 || !tiles) return e;

@@ -82,3 +82,25 @@ def test_derivative_of_the_raised_cosine():
         g = to_np(darb.darb_render_bwd(proj, 1, bins, cam, kp, 8, img, dl))[0].astype(np.float64)
         want = 8 * float(A) * dF / F
         assert abs(g[0] / g[5] - want) <= 1.6e-6 * abs(want), (q, g[0] / g[5], want)
+
+
+def test_derivative_of_the_raised_cosine_past_its_main_lobe():
+    """A caller's q_max of 60: __sinf is off by 2^-20 at x <= 10, of |sin x| >= 0.1, and F >= 0.1 by 2^-20: 2e-5."""
+    cam, proj, bins, img, dl = _one_pixel()
+    kp = darb.darb_kernel_defaults("raised_cosine")
+    kp.q_max = 60.0
+    proj.mean2d[:] = torch.tensor([[8.5, 0.5]])
+    k, seen = np.pi / 2.5, 0
+    for q in np.linspace(5.0, 60.0, 111):
+        A = np.float32(q / 64)
+        q = 64.0 * float(A)
+        proj.conic_o[:] = torch.tensor([[float(A), 0.0, 1.0, 0.5]])
+        F, dF = 0.5 + 0.5 * np.cos(k * np.sqrt(q)), -k / 4 * np.sin(k * np.sqrt(q)) / np.sqrt(q)
+        if F < 0.1 or abs(np.sin(k * np.sqrt(q))) < 0.1:
+            continue
+        seen += 1
+        img.t_final[0, 0] = 1 - 0.5 * F
+        g = to_np(darb.darb_render_bwd(proj, 1, bins, cam, kp, 8, img, dl))[0].astype(np.float64)
+        want = 8 * float(A) * dF / F
+        assert abs(g[0] / g[5] - want) <= 2e-5 * abs(want), (q, g[0] / g[5], want)
+    assert seen > 40
