@@ -106,8 +106,9 @@ inline Cam make_cam(const darb_camera &c) {
 // [0, pi], exp on [-4.5, 0]), so the hardware approximations (__cosf, __expf, __sincosf:
 // absolute error below 4e-7 there) are accurate enough; the sinc uses its Taylor series in
 // x^2 to the x^14 term (truncation error below 3e-7 on [0, pi]).
-// kernel_F is written with explicit intrinsics so that its rounding never depends on how the
-// compiler contracts the surrounding code: forward and backward must get the same alpha.
+// They are written with explicit intrinsics so that their rounding never depends on how the compiler
+// contracts the surrounding code: forward and backward must get the same alpha.  The Gaussian, the half-cosine,
+// the sinc and the parabola are in render.cu, on pairs of pixels; kernel_F has the others.
 
 // Parameters of the generic member (kind DARB_GENERIC): F = base(u), u = q^(beta/2) / xi.
 struct KernelSpec {
@@ -169,21 +170,9 @@ __device__ __forceinline__ float sqrt_newton(float q) {
 
 // exp(-q / 2) = 2^(-q / (2 ln 2))
 constexpr float kHalfLog2e = 0.72134752044448170368f;
-template <> __device__ __forceinline__ float kernel_F<DARB_GAUSSIAN>(float q, const KernelSpec &) {
-    return ex2_ftz(__fmul_rn(q, -kHalfLog2e));
-}
-
-template <> __device__ __forceinline__ float kernel_F<DARB_HALF_COSINE>(float q, const KernelSpec &) {
-    return __cosf(__fmul_rn(q, kPi / 18.0f));
-}
 
 template <> __device__ __forceinline__ float kernel_F<DARB_RAISED_COSINE>(float q, const KernelSpec &) {
     return __fmaf_rn(0.5f, __cosf(__fmul_rn(sqrt_newton(q), kPi / 2.5f)), 0.5f);
-}
-
-template <> __device__ __forceinline__ float kernel_F<DARB_MOD_SINC>(float q, const KernelSpec &) {
-    // x = pi sqrt(q) / 3, so x^2 = (pi^2 / 9) q; sin(x)/x >= 0 on the main lobe
-    return fmaxf(sinc_series(__fmul_rn(q, kPi * kPi / 9.0f)), 0.0f);
 }
 
 template <> __device__ __forceinline__ float kernel_F<DARB_INV_QUADRIC>(float q, const KernelSpec &) {
@@ -192,10 +181,6 @@ template <> __device__ __forceinline__ float kernel_F<DARB_INV_QUADRIC>(float q,
 
 template <> __device__ __forceinline__ float kernel_F<DARB_INV_MULTIQUADRIC>(float q, const KernelSpec &) {
     return rsqrt_ftz(__fadd_rn(1.0f, q));
-}
-
-template <> __device__ __forceinline__ float kernel_F<DARB_PARABOLA>(float q, const KernelSpec &) {
-    return __fmaf_rn(q, -1.0f / 9.0f, 1.0f);
 }
 
 // The generic member.  u = q / xi exactly when beta = 2, sqrt(q) / xi when beta = 1, else
@@ -419,28 +404,11 @@ __device__ __forceinline__ uint32_t instance_tile(float2 mu, float4 co, const in
     return instance_tile_p(span_prepare(mu.x, mu.y, co.x, co.y, co.z, sc.qmax), r, l, tiles_x, sc);
 }
 
-// The support test on q: 0 <= q <= q_max (q < q_max when strict).
-__device__ __forceinline__ bool in_support(float q, float qmax, bool strict) {
-    return q >= 0.0f && (strict ? q < qmax : q <= qmax);
-}
-
-// The same test with the strictness folded into the limit once: for floats, q < q_max exactly
-// when q <= the float just below q_max, so in_support(q, qmax, strict) equals
-// in_support_lim(q, support_limit(qmax, strict)) for every q (q_max positive and finite, as
-// the boundary checks).
+// The support test on q is 0 <= q <= q_max, q < q_max when strict.  The strictness is folded into the limit
+// once: for floats q < q_max exactly when q <= the float just below q_max (positive and finite, as the
+// boundary checks).
 __device__ __forceinline__ float support_limit(float qmax, bool strict) {
     return strict ? __uint_as_float(__float_as_uint(qmax) - 1u) : qmax;
-}
-__device__ __forceinline__ bool in_support_lim(float q, float qlim) { return q >= 0.0f && q <= qlim; }
-
-// q = dx (A dx + 2B dy) + (C dy) dy as a fixed FP32 sequence (no contraction beyond the
-// two explicit fused multiply-adds), shared by forward and backward so both take the
-// same support decision.  B2 = 2B (exact).
-__device__ __forceinline__ float conic_q(float dx, float dy, float A, float B2, float C) {
-    const float e = __fmul_rn(B2, dy);
-    const float g = __fmaf_rn(A, dx, e);
-    const float h = __fmul_rn(__fmul_rn(C, dy), dy);
-    return __fmaf_rn(dx, g, h);
 }
 
 // ---------------------------------------------------------------------------

@@ -36,7 +36,7 @@ struct FwdShape {
     static constexpr int TILE = TILE_, SUB = SUB_, PIX = PIX_;
     static constexpr int NT = SUB * SUB / PIX;  // threads per CTA = records per batch
     static constexpr int PARTS = (TILE / SUB) * (TILE / SUB);
-    static constexpr int LX = SUB == 32 || (SUB == 16 && PIX == 4) ? 16 : 8, LY = 32 / LX;
+    static constexpr int LX = SUB == 16 && PIX == 4 ? 16 : 8, LY = 32 / LX;
     static constexpr int BH = LY * PIX, BX = SUB / LX;  // rows of a warp's block, blocks side by side
     static_assert(BH <= SUB && SUB % BH == 0, "blocks tile the square");
     __device__ static int column() { return (int)((threadIdx.x >> 5) % BX) * LX + (int)(threadIdx.x & 31) % LX; }
@@ -54,10 +54,9 @@ template <int TILE> struct FwdOf { using S = FwdShape<TILE, TILE == 8 ? 8 : 16, 
 // its views' lists are short and half the warps then fetch items and records).
 template <int TILE> struct BatchOf { using S = FwdShape<TILE, TILE == 8 ? 8 : 16, TILE == 8 ? 2 : 4>; };
 
-// Lane arithmetic on one value or on a pair (the packed two-lane FP32 instructions of sm_100+, which
-// round each lane as the scalar form does).
-template <int L> struct Lanes;
-template <> struct Lanes<2> {
+// Arithmetic on a pair of values (the packed two-lane FP32 instructions of sm_100+, which round each lane
+// as the scalar form does).
+struct Pair {
     using T = float2;
     static __device__ __forceinline__ T dup(float a) { return make_float2(a, a); }
     static __device__ __forceinline__ T mul(T a, T b) { return __fmul2_rn(a, b); }
@@ -66,20 +65,29 @@ template <> struct Lanes<2> {
     static __device__ __forceinline__ float &at(T &v, int l) { return l ? v.y : v.x; }
 };
 
-// kernel_F on every lane: the multiplications in front of the special functions, and the whole sinc
-// series, on pairs.  The same operations as kernel_F, so the same bits.
-template <int KIND, int L>
-__device__ __forceinline__ typename Lanes<L>::T kernel_F_lanes(typename Lanes<L>::T q, const KernelSpec &ks) {
-    using V = Lanes<L>;
-    typename V::T r = q;
+// q = dx (A dx + 2B dy) + (C dy) dy as a fixed FP32 sequence, for a record (B2 = 2B, exact) and a pair of
+// pixels of one column.  Forward and backward both call it, so that they take the same support
+// decision.
+__device__ __forceinline__ float2 conic_q(float2 dx, float2 dy, float2 A, float2 B2, float2 C) {
+    using V = Pair;
+    const float2 g = V::fma(A, dx, V::mul(B2, dy));
+    return V::fma(dx, g, V::mul(V::mul(C, dy), dy));
+}
+
+// The profile F of a pair of values: the multiplications in front of the special functions, and the whole
+// sinc series (sin(x)/x >= 0 on the main lobe, x^2 = pi^2 q / 9), on the pair, the other kernels by lane.
+template <int KIND>
+__device__ __forceinline__ float2 kernel_F_pair(float2 q, const KernelSpec &ks) {
+    using V = Pair;
+    float2 r = q;
     if constexpr (KIND == DARB_GAUSSIAN || KIND == DARB_HALF_COSINE) {
         r = V::mul(q, V::dup(KIND == DARB_GAUSSIAN ? -kHalfLog2e : kPi / 18.0f));
 #pragma unroll
-        for (int l = 0; l < L; ++l) V::at(r, l) = KIND == DARB_GAUSSIAN ? ex2_ftz(V::at(r, l)) : __cosf(V::at(r, l));
+        for (int l = 0; l < 2; ++l) V::at(r, l) = KIND == DARB_GAUSSIAN ? ex2_ftz(V::at(r, l)) : __cosf(V::at(r, l));
     } else if constexpr (KIND == DARB_PARABOLA) {
         r = V::fma(q, V::dup(-1.0f / 9.0f), V::dup(1.0f));
     } else if constexpr (KIND == DARB_MOD_SINC) {
-        const typename V::T u = V::mul(q, V::dup(kPi * kPi / 9.0f));
+        const float2 u = V::mul(q, V::dup(kPi * kPi / 9.0f));
         r = V::fma(u, V::dup(1.0f / 1307674368000.0f), V::dup(-1.0f / 6227020800.0f));
         r = V::fma(r, u, V::dup(1.0f / 39916800.0f));
         r = V::fma(r, u, V::dup(-1.0f / 362880.0f));
@@ -88,10 +96,10 @@ __device__ __forceinline__ typename Lanes<L>::T kernel_F_lanes(typename Lanes<L>
         r = V::fma(r, u, V::dup(1.0f / 6.0f));
         r = V::fma(r, V::mul(u, V::dup(-1.0f)), V::dup(1.0f));
 #pragma unroll
-        for (int l = 0; l < L; ++l) V::at(r, l) = fmaxf(V::at(r, l), 0.0f);
+        for (int l = 0; l < 2; ++l) V::at(r, l) = fmaxf(V::at(r, l), 0.0f);
     } else {
 #pragma unroll
-        for (int l = 0; l < L; ++l) V::at(r, l) = kernel_F<KIND>(V::at(q, l), ks);
+        for (int l = 0; l < 2; ++l) V::at(r, l) = kernel_F<KIND>(V::at(q, l), ks);
     }
     return r;
 }
@@ -220,9 +228,10 @@ __device__ __forceinline__ void render_tile_fwd(int item, FwdSmem<S::NT> &sm,
                                                 int W, int H, int tiles_x, float qmax, int strict,
                                                 const KernelSpec &ks, SinkFn sink, const L1Out &l1 = L1Out{},
                                                 float *s_l1 = nullptr, float *l1_sum = nullptr) {
-    constexpr int TILE = S::TILE, NT = S::NT, PIX = S::PIX, L = PIX % 2 == 0 ? 2 : 1, NV = PIX / L;  // NV groups of L lanes
-    using V = Lanes<L>;
-    using VT = typename V::T;
+    constexpr int TILE = S::TILE, NT = S::NT, PIX = S::PIX, L = 2, NV = PIX / L;  // NV pairs
+    using V = Pair;
+    using VT = V::T;
+    static_assert(PIX % L == 0, "whole pairs");
     static_assert(NT % STEP == 0, "a full batch is whole steps");
     const int tile = item / S::PARTS, part = item % S::PARTS;
     const int px = (tile % tiles_x) * TILE + part % (TILE / S::SUB) * S::SUB + S::column();
@@ -291,9 +300,8 @@ __device__ __forceinline__ void render_tile_fwd(int item, FwdSmem<S::NT> &sm,
 #pragma unroll
                     for (int v = 0; v < NV; ++v) {
                         const VT dy = V::add(y, nfpy[v]);
-                        const VT g = V::fma(A, dx, V::mul(B2, dy));  // conic_q
-                        VT q = V::fma(dx, g, V::mul(V::mul(Cc, dy), dy));
-                        VT a = V::mul(o, kernel_F_lanes<KIND, L>(q, ks));
+                        VT q = conic_q(dx, dy, A, B2, Cc);
+                        VT a = V::mul(o, kernel_F_pair<KIND>(q, ks));
                         bool use[L];
 #pragma unroll
                         for (int l = 0; l < L; ++l) {
@@ -751,8 +759,7 @@ k_render_bwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ valu
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
                     const float2 dy = __fadd2_rn(y, nfpy[v]);
-                    const float2 e = __ffma2_rn(A, dx, __fmul2_rn(B2, dy));  // conic_q
-                    const float2 qr = __ffma2_rn(dx, e, __fmul2_rn(__fmul2_rn(Cc, dy), dy));
+                    const float2 qr = conic_q(dx, dy, A, B2, Cc);
                     // outside the support the profile is taken at its limit: finite, so that the pair's zero
                     // weight leaves the sums alone (as unsigned words negative values lie above the limit too)
                     const uint32_t q0 = __float_as_uint(qr.x), q1 = __float_as_uint(qr.y);
@@ -765,7 +772,7 @@ k_render_bwd(const uint2 *__restrict__ ranges, const uint32_t *__restrict__ valu
                             generic_both(q.y, ks, F.y, dF.y);
                         }
                     } else {
-                        F = kernel_F_lanes<KIND == kRaisedCosineWide ? DARB_RAISED_COSINE : KIND, 2>(q, ks);
+                        F = kernel_F_pair<KIND == kRaisedCosineWide ? DARB_RAISED_COSINE : KIND>(q, ks);
                         dF = kernel_dF2<KIND>(q, F);
                     }
                     const float2 of = __fmul2_rn(o, F);
