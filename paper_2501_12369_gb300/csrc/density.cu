@@ -235,7 +235,7 @@ __device__ __forceinline__ void zero_moments(const darb_adam_state &s, uint32_t 
 // workspace).  It lists its survivors, clones and split parents in shared memory; the rows of
 // each list are consecutive in the output, so every array is then copied as one flat range.
 // HBM-bound: with one thread copying each row, 32 lanes wrote 32 different rows at a time and the
-// kernel took 1250 us (1M splats, SH degree 3, 1.6 GB), now 277 us (0.78 of the measured copy rate).
+// kernel took 1250 us (1M splats, SH degree 3, 1.46 GB), now 277 us (0.78 of the measured copy rate).
 template <int K3>
 __global__ void __launch_bounds__(kDenThreads)
 k_densify_scatter(int n, DenIO io, const float *__restrict__ accum, const float *__restrict__ count,

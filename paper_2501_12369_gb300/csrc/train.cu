@@ -48,7 +48,7 @@ k_l1_loss(const float *__restrict__ image, const float *__restrict__ target, int
 // thread's lanes issued before the first update.  HBM-bound; as a launch per group (and scalar lanes
 // for the SH rows whose length is no multiple of 4) the small groups ran at half the copy rate
 // and a small state was five launches: 243 -> 232 us at 1M splats,
-// degree 3 (1.63 GB at 7.0 TB/s); with the gradients before it, degree 2 320 -> 220 us, degree 0 111 -> 101.
+// degree 3 (1684 B a splat; part of the gradients is still in L2); with the gradients before it, degree 2 320 -> 220 us, degree 0 111 -> 101.
 constexpr int kAdamThreads = 256, kAdamLanes = 2;
 constexpr int kAdamBlock = kAdamThreads * kAdamLanes * 4;  // floats per block
 
