@@ -280,7 +280,8 @@ darb_status darb_render_fwd_l1(const darb_projected *proj, const darb_binning *b
  * gradients.  n: number of splats.  dL_dimage: device [3][H][W].  grad2d: device [n][12],
  * zeroed by the callee,
  * per splat (d mu'x, d mu'y, dA, dB, dC, d opacity, dr, dg, db, 0, 0, 0).  The alpha
- * clamp at 0.99 has zero derivative. */
+ * clamp at 0.99 has zero derivative.  Sums over tiles are added in an order that varies from run
+ * to run; those of the conic are rounded once for splats of eight tiles or more. */
 darb_status darb_render_bwd(const darb_projected *proj, int32_t n, const darb_binning *bins,
                             const darb_camera *cam, const darb_kernel_params *kparams,
                             int32_t tile, const darb_image *fwd, const float *dL_dimage,

@@ -130,6 +130,7 @@ cudaError_t launch_render_fwd(int kind, int tile, int tiles_x, int tiles_y, cons
                               float *image, float *t_final, uint32_t *last, uint32_t *n_contrib,
                               cudaStream_t st, const float *l1_target = nullptr, float *l1_dL = nullptr,
                               float *l1_loss = nullptr);
+// tiles: member tiles of each of the n splats; the conic's sums of a splat with many are kept whole.
 cudaError_t launch_render_bwd(int kind, int n, const uint32_t *tiles, int tile, int tiles_x, int tiles_y, const uint32_t *ranges,
                               const uint32_t *values, const float2 *mean2d, const float4 *conic_o,
                               const float *rgb, const Cam &cam, float qmax, int strict, const KernelSpec &ks,
